@@ -306,6 +306,7 @@ constexpr int kRowMaxThreads = 512;  // one-thread-per-row / per-edge kernels: 1
 constexpr int kHighMaxBlock = 288;   // element sweep: whole elements, at most this many nodes per block
 constexpr int kHighDefaultCap = 288;  // the element block of an untuned schedule
 constexpr int kLsfixThreads = 128;
+constexpr long long kLsfixMaxBlocks = 152 * 16;  // 16 blocks for each SM: 311,296 searches at once
 
 // The launch schedule: threads per block of each one-thread-per-row kernel (KN_EDGE: per edge), the
 // largest element block of the element sweep (whole elements, <= kHighMaxBlock nodes), and how many
@@ -354,8 +355,11 @@ inline long long kernel_blocks(int k, const Dev& D, const Sched& sc) {
       // The queue length is only known on the device.  The grid covers the entries at lsfix_slots per
       // thread (a deferred search per thread unless more than that share of the entries defer, when the
       // threads take a few each), and its blocks beyond the queue return before loading their context.
+      // Never more blocks than kLsfixMaxBlocks: beyond that the launch is paid for in empty blocks (172,000
+      // of them at Q2 1024^2, where the queue fills 700).
       const long long per_block = (long long)kLsfixThreads * sc.lsfix_slots;
-      return D.n == 0 ? 0 : ((long long)D.nnz + D.nb + per_block - 1) / per_block;
+      const long long cover = D.n == 0 ? 0 : ((long long)D.nnz + D.nb + per_block - 1) / per_block;
+      return cover < kLsfixMaxBlocks ? cover : kLsfixMaxBlocks;
     }
     default: return (row_slots(D, (sc.slices >> k) & 1) + sc.bt[k] - 1) / sc.bt[k];
   }
@@ -756,6 +760,15 @@ __device__ __forceinline__ double dot(const double* a, const double* b) {
   return s;
 }
 
+// The same on the FP64 pipe, for the line searches (mulp).
+template <int DIM>
+__device__ __forceinline__ double dot_fp64(const double* a, const double* b) {
+  double s = __dmul_rn(a[0], b[0]);
+#pragma unroll
+  for (int k = 1; k < DIM; ++k) s = fma(a[k], b[k], s);
+  return s;
+}
+
 template <int DIM>
 __device__ __forceinline__ double internal_energy(const double* U) {
   const double m2 = dot<DIM>(U + 1, U + 1);
@@ -861,11 +874,9 @@ struct LsRow {
 template <int DIM>
 __device__ __forceinline__ void ls_row(const Dev& D, LsRow<DIM>& c, const double* U0, double rmin, double rmax,
                                        double smin) {
-  double m2 = 0.0;
 #pragma unroll
   for (int q = 0; q < DIM + 2; ++q) c.U0[q] = U0[q];
-#pragma unroll
-  for (int k = 0; k < DIM; ++k) m2 += U0[1 + k] * U0[1 + k];
+  const double m2 = dot_fp64<DIM>(U0 + 1, U0 + 1);
   c.rmin = rmin;
   c.rmax = rmax;
   c.smin = smin;
@@ -901,50 +912,25 @@ __device__ __forceinline__ double ls_psi(const Dev& D, const double* U0, const d
 #pragma unroll
   for (int q = 0; q < DIM + 2; ++q) V[q] = fma(s, A[q], U0[q]);
   if (!(V[0] > 0.0)) return -1.0;
-  double m2 = 0.0;
-#pragma unroll
-  for (int k = 0; k < DIM; ++k) m2 += V[1 + k] * V[1 + k];
+  const double m2 = dot_fp64<DIM>(V + 1, V + 1);
   double irho;
   double rg = rho_pow_gamma<false>(D, V[0], &irho);
   return fma(-smin, rg, fma(-sf::mul_pow2(m2, -1), irho, V[DIM + 1]));
 }
 
-// d psi / d s
-template <int DIM>
-__device__ __forceinline__ double ls_dpsi(const Dev& D, const double* U0, const double* A, double s, double smin) {
-  double V[DIM + 2];
-#pragma unroll
-  for (int q = 0; q < DIM + 2; ++q) V[q] = fma(s, A[q], U0[q]);
-  double mA = 0.0, m2 = 0.0;
-#pragma unroll
-  for (int k = 0; k < DIM; ++k) {
-    mA += V[1 + k] * A[1 + k];
-    m2 += V[1 + k] * V[1 + k];
-  }
-  double irho;
-  double rg = rho_pow_gamma<false>(D, V[0], &irho);
-  double deps = A[DIM + 1] - mA * irho + 0.5 * m2 * A[0] * irho * irho;
-  return deps - smin * D.gamma * rg * irho * A[0];
-}
-
-// psi(s) and d psi / d s together (the two share the state, rho^gamma and 1/rho), each computed as
-// ls_psi and ls_dpsi compute it.
+// psi(s), computed as ls_psi computes it, and d psi / d s (the two share the state, rho^gamma and 1/rho).
 template <int DIM>
 __device__ __forceinline__ double ls_psi_dpsi(const Dev& D, const double* U0, const double* A, double s, double smin,
                                               double* dpsi) {
   double V[DIM + 2];
 #pragma unroll
   for (int q = 0; q < DIM + 2; ++q) V[q] = fma(s, A[q], U0[q]);
-  double mA = 0.0, m2 = 0.0;
-#pragma unroll
-  for (int k = 0; k < DIM; ++k) {
-    mA += V[1 + k] * A[1 + k];
-    m2 += V[1 + k] * V[1 + k];
-  }
+  const double mA = dot_fp64<DIM>(V + 1, A + 1), m2 = dot_fp64<DIM>(V + 1, V + 1);
   double irho;
   double rg = rho_pow_gamma<false>(D, V[0], &irho);
-  double deps = A[DIM + 1] - mA * irho + 0.5 * m2 * A[0] * irho * irho;
-  *dpsi = deps - smin * D.gamma * rg * irho * A[0];
+  // A_E - mA / rho + (A_rho / rho) (|m|^2 / (2 rho) - gamma s_min rho^gamma)
+  *dpsi = fma(__dmul_rn(A[0], irho), fma(sf::mul_pow2(m2, -1), irho, -__dmul_rn(__dmul_rn(smin, D.gamma), rg)),
+              fma(-mA, irho, A[DIM + 1]));
   if (!(V[0] > 0.0)) return -1.0;
   return fma(-smin, rg, fma(-sf::mul_pow2(m2, -1), irho, V[DIM + 1]));
 }
@@ -995,11 +981,9 @@ __device__ __forceinline__ bool ls_certified(const Dev& D, const LsRow<DIM>& c, 
 // Largest l in [0, 1] with U0 + l P in B_i, P = w A (Sec. 5.4, eq. (ConvexScheme), Lemma
 // ConsInvariants), in two parts.  The head takes the closed form for the density bounds and decides the
 // common cases: the entropy constraint holds at l_rho (proved by the FP32 certificate, else by psi in FP64),
-// or psi(0) < 0 (roundoff) and l = 0.  It returns false when psi(l_rho) < 0 <= psi(0); then the tail runs
-// a bracketed iteration on the concave psi from [0, l_rho]: the chord root stays feasible, the tangent root
-// from the infeasible end stays infeasible, and a bisection follows every iteration that has not halved the
-// bracket; it stops when the bracket is at most ls_tol wide and returns the feasible end.  The FP32 certificate only skips FP64
-// evaluations whose outcome it proves; the result is that of the FP64 search.
+// or psi(0) < 0 (roundoff) and l = 0.  It returns false when psi(l_rho) < 0 <= psi(0): then the tail looks for
+// the root in between and returns a feasible point within ls_tol, or psi's rounding, of it.  The FP32
+// certificate only skips FP64 evaluations whose outcome it proves.
 template <int DIM>
 __device__ __forceinline__ bool line_search_head(const Dev& D, const LsRow<DIM>& c, const double* A, double w,
                                                  float wf, double* l_out, double* fb_out) {
@@ -1014,7 +998,7 @@ __device__ __forceinline__ bool line_search_head(const Dev& D, const LsRow<DIM>&
   double l = 1.0;
   float sf = wf;
   if (!inside) {
-    const double Pr = w * A[0];
+    const double Pr = __dmul_rn(w, A[0]);
     if (c.U0[0] + Pr < c.rmin) l = (c.rmin - c.U0[0]) / Pr;
     if (c.U0[0] + Pr > c.rmax) l = (c.rmax - c.U0[0]) / Pr;
     if (!(l > 0.0)) l = 0.0;
@@ -1033,43 +1017,171 @@ __device__ __forceinline__ bool line_search_head(const Dev& D, const LsRow<DIM>&
   return false;
 }
 
+// Root of psi(t) on (0, l) in FP32, psi(0) = psi0 >= 0 > psi(l), t in units of P = w A: Newton steps from the
+// infeasible end on the concave psi in the differenced form of ls_certified (which keeps small increments
+// from drowning in |U0|), so that the iterates fall monotonically onto the root.  Good to about 1e-6 of t;
+// 0 or NaN where it fails (an input outside the FP32 range, no root before the last step).
 template <int DIM>
-__device__ double line_search_tail(const Dev& D, const LsRow<DIM>& c, const double* A, double w,
-                                                double l, double fb) {
-  const double* U0 = c.U0;
-  const double smin = c.smin;
-  double fa = c.psi0;
-  double a = 0.0, b = l;
-  // the slope at b, kept while b stays: the tangent point, which usually becomes the next b, is evaluated
-  // with its slope; a b set by the chord or the bisection takes it afresh at the next iteration
-  double dfb = 0.0;
-  bool fresh = false;
-  for (int it = 0; it < D.ls_maxit && b - a > D.ls_tol; ++it) {
-    const double width = b - a;
-    double ts = a + (b - a) * fa / (fa - fb);
-    if (!fresh) dfb = w * ls_dpsi<DIM>(D, U0, A, b * w, smin);
-    fresh = true;
-    double tn = dfb < 0.0 ? b - fb / dfb : b;
-    if (ts > a && ts < b) {
-      double fs = ls_psi<DIM>(D, U0, A, ts * w, smin);
-      if (fs >= 0.0) { a = ts; fa = fs; } else { b = ts; fb = fs; fresh = false; }
-    }
-    if (tn > a && tn < b) {
-      double dn;
-      double fn = ls_psi_dpsi<DIM>(D, U0, A, tn * w, smin, &dn);
-      if (fn >= 0.0) { a = tn; fa = fn; } else { b = tn; fb = fn; dfb = w * dn; fresh = true; }
-    }
-    // Near the root psi is evaluated below its rounding resolution (a change of t by an ulp leaves
-    // U0 + t P unchanged), and the chord and tangent points then creep towards one end while the other
-    // stays put: when the bracket has not halved, bisect, so that it always shrinks to ls_tol.
-    if (b - a > 0.5 * width) {
-      double tm = a + 0.5 * (b - a);
-      if (!(tm > a && tm < b)) break;
-      double fm = ls_psi<DIM>(D, U0, A, tm * w, smin);
-      if (fm >= 0.0) { a = tm; fa = fm; } else { b = tm; fb = fm; fresh = false; }
-    }
+__device__ __forceinline__ float ls_root_f32(const Dev& D, const double* U0, const double* A, double w, double smin,
+                                             double l, double psi0) {
+  const float P0 = (float)(w * A[0]), PE = (float)(w * A[DIM + 1]), r0 = (float)U0[0], ir0 = 1.f / r0;
+  float mP = 0.f, PP = 0.f, m0sq = 0.f;
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) {
+    const float m0 = (float)U0[1 + k], Pm = (float)(w * A[1 + k]);
+    mP = fmaf(m0, Pm, mP);
+    PP = fmaf(Pm, Pm, PP);
+    m0sq = fmaf(m0, m0, m0sq);
   }
-  return a;
+  // s_min rho0^gamma = E0 - |m0|^2 / (2 rho0) - psi(0).  Sums of products are written as explicit fused
+  // operations, so that every instantiation rounds alike.
+  const float psi0f = (float)psi0;
+  const float sg0 = fmaf(__fmul_rn(-0.5f, m0sq), ir0, (float)U0[DIM + 1]) - psi0f;
+  float t = (float)l;
+#pragma unroll 1
+  for (int it = 0; it < 12; ++it) {
+    const float a = __fmul_rn(t, P0), ir = 1.f / (r0 + a);
+    const float dm2 = __fmul_rn(t, fmaf(t, PP, 2.f * mP));  // |m(t)|^2 - |m0|^2
+    const float dK = __fmul_rn(__fmul_rn(fmaf(r0, dm2, -__fmul_rn(a, m0sq)), 0.5f * ir0), ir);
+    const float ex = expm1f(__fmul_rn(D.gamma_f, log1pf(__fmul_rn(a, ir0))));
+    const float f = fmaf(-sg0, ex, fmaf(t, PE, psi0f - dK));
+    const float q = fmaf(0.5f * (m0sq + dm2), ir, -__fmul_rn(D.gamma_f, fmaf(sg0, ex, sg0)));
+    const float df = fmaf(__fmul_rn(q, ir), P0, fmaf(-fmaf(t, PP, mP), ir, PE));
+    const float step = __fdiv_rn(f, df);
+    t -= step;
+    if (!(fabsf(step) > 1e-6f * t)) break;
+  }
+  return t;
+}
+
+// What psi's own rounding leaves open, relative to E: its terms are at most E in size, each good to an ulp
+// or so.
+constexpr double kPsiRounding = 2.220446049250313e-16;
+
+// The search of an entry whose head found psi(l_rho) < 0 <= psi(0), from the same values.  Newton steps in
+// FP64 from the FP32 root reach the rounding of psi in two or three evaluations; every evaluated point
+// narrows the bracket [a, b] of feasible and infeasible ends.  The search ends where the step is at most
+// half the tolerance, or where psi or the bracket is below psi's own rounding (then its sign, not its
+// size, is all there is): at that point when it is feasible, else at one just before it that is.  A step that
+// leaves the bracket, or does not settle in a few, hands over to the plain bracketed iteration (chord
+// root, tangent root from the infeasible end, and a bisection where the bracket has not halved), which is
+// also what a caller gets who allows fewer than 8 iterations.
+//
+// What bounds it is the length of the chain: every search is one thread, its evaluations follow one
+// another, and each is some 25 dependent FP64 operations of 64 clocks.  The plain iteration takes 20 to
+// 60 of them, this one about 4.  All of them go through one copy of the evaluation, chosen by a phase:
+// lanes of a warp evaluate together whatever they do next, and the code a warp has to fetch cold, which
+// on small meshes takes longer than running it, stays short.  Per launch of k_lsfix, against the plain
+// iteration: 110 -> 24 us for 1,435 searches (Q2, 33 x 47 quads), 1,207 -> 238 us for 493,000 (Q1,
+// 48 x 40 x 44 hexahedra), 316 -> 66 us for 91,000 (Q2, 1024^2).
+template <int DIM>
+__device__ __forceinline__ double line_search_tail(const Dev& D, const double* U0, const double* A, double w,
+                                                   double rmin, double rmax, double smin) {
+  enum { kZero, kNewton, kBack, kEnd, kChord, kTangent, kMiddle };
+  double l = 1.0;  // the density bounds in closed form, as in the head
+  {
+    const double Pr = __dmul_rn(w, A[0]);
+    if (U0[0] + Pr < rmin) l = (rmin - U0[0]) / Pr;
+    if (U0[0] + Pr > rmax) l = (rmax - U0[0]) / Pr;
+    if (!(l > 0.0)) l = 0.0;
+    if (l > 1.0) l = 1.0;
+  }
+  double a = 0.0, b = l, fa = 0.0, fb = 0.0, dfb = 0.0;
+  double t = 0.0, t0 = 0.0, back = 0.0, width = 0.0, tn = 0.0;
+  int phase = kZero, count = 0;
+  bool have_b = false;  // psi(b) and its slope are known
+  for (;;) {
+    double d;
+    const double f = ls_psi_dpsi<DIM>(D, U0, A, t * w, smin, &d);
+    d *= w;
+    const bool ok = f >= 0.0;
+    if (phase == kZero) {
+      if (!ok) return 0.0;
+      fa = f;
+      t = D.ls_maxit >= 8 ? (double)ls_root_f32<DIM>(D, U0, A, w, smin, l, f) : 0.0;
+      phase = kNewton;
+      if (t > a && t < b) continue;
+      phase = kEnd;
+      t = b;
+      continue;
+    }
+    if (phase == kEnd && ok) return b;
+    if (ok) {
+      a = t;
+      fa = f;
+    } else {
+      b = t;
+      fb = f;
+      dfb = d;
+      have_b = true;
+    }
+    if (phase == kNewton && d < 0.0) {
+      const double id = 1.0 / d, step = __dmul_rn(f, id);
+      const double noise = -kPsiRounding * fma(t * w, A[DIM + 1], U0[DIM + 1]) * id;
+      if (b - a <= fmax(D.ls_tol, 4.0 * noise)) return a;
+      const double thr = fmax(0.5 * D.ls_tol, noise);
+      if (fabs(step) <= thr) {
+        if (ok) return t;
+        back = fabs(step) + thr;
+        t0 = t;
+        t = t0 - back;
+        if (!(t > a)) return a;
+        phase = kBack;
+        count = 0;
+        continue;
+      }
+      t -= step;
+      if (t > a && t < b && ++count < 8) continue;
+    }
+    if (phase == kBack) {
+      if (ok) return t;
+      back *= 4.0;
+      t = t0 - back;
+      if (!(t > a)) return a;  // the bracket is no wider than what the step and the rounding leave open
+      if (++count < 3) continue;
+    }
+    if (phase <= kBack) {  // the Newton steps did not settle: on to the plain iteration
+      phase = kEnd;
+      if (!have_b) {
+        t = b;
+        continue;
+      }
+    }
+    if (phase == kEnd) {
+      count = 0;
+      phase = kMiddle;
+      width = 2.0 * (b - a);  // (the bisection below is for an iteration that has been run)
+    } else {
+      ++phase;  // the next of chord, tangent, middle that lies inside the bracket, then the next iteration
+    }
+    if (phase == kTangent) {
+      t = tn;
+      if (t > a && t < b) continue;
+      phase = kMiddle;
+    }
+    if (phase == kMiddle && b - a > 0.5 * width) {
+      // Near the root psi is evaluated below its rounding resolution (a change of t by an ulp leaves
+      // U0 + t P unchanged), and the chord and tangent points then creep towards one end while the other
+      // stays put: when the bracket has not halved, bisect, so that it always shrinks to ls_tol.
+      t = a + 0.5 * (b - a);
+      if (!(t > a && t < b)) return a;
+      continue;
+    }
+    // the next iteration
+    if (count >= D.ls_maxit || !(b - a > D.ls_tol)) return a;
+    ++count;
+    width = b - a;
+    tn = dfb < 0.0 ? b - fb / dfb : b;
+    phase = kChord;
+    t = a + (b - a) * fa / (fa - fb);
+    if (t > a && t < b) continue;
+    phase = kTangent;
+    t = tn;
+    if (t > a && t < b) continue;
+    phase = kMiddle;
+    t = a + 0.5 * (b - a);  // neither point lies inside: the bracket has not halved
+    if (!(t > a && t < b)) return a;
+  }
 }
 
 // The searches that need the tail are rare (well under 1% of the entries) but take ~10 iterations, and a

@@ -95,8 +95,7 @@ __global__ void __maxnreg__(72) k_limit2(Src src, int sliced, int last) {
 
 // The deferred line searches of one limiter pass (pass 0: from U^L with P = A / (kappa_i m_i), written to
 // l1; pass 1: from U^(1) with P = (1 - l1_ij) A / (kappa_i m_i), written to l2).  One thread per queued
-// entry, grid-stride over the queue: every lane runs a bracketed iteration.  The row context, l_rho and
-// psi(l_rho) are recomputed from the same stored values by the same code as in the queuing kernel.
+// entry, grid-stride over the queue.
 template <int DIM, class Src>
 __device__ __forceinline__ void lsfix_body(const Src& src, int pass) {
   constexpr int M = DIM + 2;
@@ -124,10 +123,7 @@ __device__ __forceinline__ void lsfix_body(const Src& src, int pass) {
     }
     double w = D.inv_km[i];
     if (pass == 1) w = (1.0 - (bnd ? S.l1B[e] : pmin(S.l1[e], S.l1[D.tr[e]]))) * w;
-    LsRow<DIM> ls;
-    ls_row<DIM>(D, ls, U0, S.bounds[i], S.bounds[n + i], S.bounds[2 * n + i]);
-    double l, fb;
-    if (!line_search_head<DIM>(D, ls, A, w, d2f_fast(w), &l, &fb)) l = line_search_tail<DIM>(D, ls, A, w, l, fb);
+    const double l = line_search_tail<DIM>(D, U0, A, w, S.bounds[i], S.bounds[n + i], S.bounds[2 * n + i]);
     double* dst = pass == 0 ? (bnd ? S.l1B : S.l1) : (bnd ? S.l2B : S.l2);
     dst[e] = l;
   }
