@@ -102,9 +102,10 @@ struct Arena {
   X(rbeg, int, n) X(rend, int, n) X(sten, int, n) X(col, int, nnz) X(tr, int, nnz) X(cnorm, double, nnz) X(cn, double, dim * nnz)   \
   X(mij, double, nnz) X(mu, double, nnz) X(mi, double, n) X(imi, double, n) X(ikm, double, n)             \
   X(rm, double, n) X(rp, double, n) X(muB, double, n) X(bptr, int, n + 1) X(bnorm, double, nb)           \
-  X(bn, double, dim * nb) X(btype, int, nb) X(borig, int, nb) X(minv, double, nel * nl * nl)             \
+  X(bn, double, dim * nb) X(btype, int, nb) X(borig, int, nb) X(bnode, int, nb) X(minv, double, nel * nl * nl)             \
   X(ee, int, ne) X(ei, int, ne) X(G, double, m * nnz) X(barR, double, nnz) X(barS, double, nnz)          \
   X(prim, double, gdg::NPRIM * n) X(dL, double, nnz) X(dB, double, nb) X(bbar, double, 2 * nb)            \
+  X(UB, double, m * nb) X(gB, double, m * nb) X(gI, double, m * nb)                                       \
   X(UL, double, m * n) X(RHSL, double, m * n) X(N, double, n) X(agg, double, 3 * n) X(A, double, m * nnz) \
   X(AB, double, m * nb) X(bounds, double, 3 * n) X(l1, double, nnz) X(l1B, double, nb) X(l2, double, nnz) \
   X(l2B, double, nb) X(U1, double, m * n) X(rem, unsigned char, n) X(flags, unsigned, 4)                 \
@@ -509,7 +510,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   }
   const int64_t ne = (int64_t)edge_e.size();
   std::vector<double> bnorm(nb), bn((size_t)dim * nb);
-  std::vector<int> btype(nb);
+  std::vector<int> btype(nb), bnode(nb);
   for (int64_t t = 0; t < nb; ++t) {
     int b = border[t];
     double c2 = 0;
@@ -517,6 +518,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
     bnorm[t] = std::sqrt(c2);
     for (int k = 0; k < dim; ++k) bn[(size_t)k * nb + t] = P->b_c[(size_t)k * nb + b] / bnorm[t];
     btype[t] = P->b_type[b];
+    bnode[t] = P->b_node[b];
   }
 
   ParamArrays pa;
@@ -558,6 +560,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
       (ce = up(o_bn, bn.data(), sizeof(double) * dim * nb)) != cudaSuccess ||
       (ce = up(o_btype, btype.data(), sizeof(int) * nb)) != cudaSuccess ||
       (ce = up(o_borig, border.data(), sizeof(int) * nb)) != cudaSuccess ||
+      (ce = up(o_bnode, bnode.data(), sizeof(int) * nb)) != cudaSuccess ||
       (ce = up(o_minv, minv_g.data(), sizeof(double) * minv_g.size())) != cudaSuccess ||
       (ce = up(o_ee, edge_e.data(), sizeof(int) * ne)) != cudaSuccess ||
       (ce = up(o_ei, edge_i.data(), sizeof(int) * ne)) != cudaSuccess ||
@@ -591,6 +594,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   D.bn = (const double*)ptr(o_bn);
   D.btype = (const int*)ptr(o_btype);
   D.borig = (const int*)ptr(o_borig);
+  D.bnode = (const int*)ptr(o_bnode);
   D.MKinv = (const double*)ptr(o_minv);
   D.ne = (int)ne;
   D.edge_e = (const int*)ptr(o_ee);
@@ -609,6 +613,9 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   S.barS = (double*)ptr(o_barS);
   S.dB = (double*)ptr(o_dB);
   S.bbar = (double*)ptr(o_bbar);
+  S.UB = (double*)ptr(o_UB);
+  S.gB = (double*)ptr(o_gB);
+  S.gI = (double*)ptr(o_gI);
   S.UL = (double*)ptr(o_UL);
   S.RHSL = (double*)ptr(o_RHSL);
   S.N = (double*)ptr(o_N);

@@ -64,7 +64,6 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   const Dev& D = c.D;
   const Scratch& S = c.S;
   const double* U = c.U;
-  const double* bdata = c.bdata;
   const ElemSlot es = element_slot(D, lb, eb);
   const int i = es.i;
   const bool valid = es.ok;
@@ -148,10 +147,9 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
         hi = pmax(hi, S.bbar[b]);
         sl = pmin(sl, S.bbar[(size_t)D.nb + b]);
       }
-      double nv[DIM], UB[M];
+      double UB[M];  // from the edge sweep
 #pragma unroll
-      for (int k = 0; k < DIM; ++k) nv[k] = D.bn[(size_t)k * D.nb + b];
-      boundary_state<DIM>(D, b, Ui, bdata, nv, UB);
+      for (int q = 0; q < M; ++q) UB[q] = S.UB[(size_t)q * D.nb + b];
       double dl = S.dB[b];
       double dd = (pmax(D.muB[i], pmin(D.c_ev * Ni, 1.0)) - 1.0) * dl;
 #pragma unroll

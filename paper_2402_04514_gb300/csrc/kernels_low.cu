@@ -178,12 +178,10 @@ __global__ void __launch_bounds__(kThreads) k_maxdt(Src src, int sliced) {
 }
 
 // The same bound inside the fused SSP-RK3 step, after the edge sweep of the step's first stage: the row
-// sums of the stored d_ij^L plus the boundary viscosities, reduced into the instance's clock.  Capped at
-// 48 registers: the row sum, which every row runs, is latency-bound and wants many warps; the boundary
-// viscosities of the few boundary rows would otherwise take 117 and spill at the cap.
+// sums of the stored d_ij^L and boundary viscosities, reduced into the instance's clock.  Capped at
+// 48 registers: the row sum is latency-bound and wants many warps.
 template <int DIM, bool MX, class Src>
 __device__ __forceinline__ void tau_body(const Src& src, int sliced) {
-  constexpr int M = DIM + 2;
   __shared__ Ctx sctx;
   int lb;
   const Ctx& c = src.get(&sctx, &lb);
@@ -197,16 +195,7 @@ __device__ __forceinline__ void tau_body(const Src& src, int sliced) {
     const int e0 = D.rbeg[i], e1 = D.sten_end[i];
 #pragma unroll 4
     for (int e = e0; e < e1; e += kEll) dsum += __ldg(S.dL + e);  // loads issued ahead of the in-order sum
-    const int b0 = D.b_ptr[i], b1 = D.b_ptr[i + 1];
-    if (b0 < b1) {
-      const size_t n = D.n;
-      const double* P = S.prim;
-      double Ui[M];
-      load_state<DIM>(c.U, D.n, i, Ui);
-      for (int b = b0; b < b1; ++b)
-        dsum += boundary_viscosity<DIM, MX>(D, b, Ui, c.bdata, P[PR_IRHO * n + i], P[PR_P * n + i], P[PR_IP * n + i],
-                                        P[PR_A * n + i], P[PR_PME * n + i]);
-    }
+    for (int b = D.b_ptr[i], b1 = D.b_ptr[i + 1]; b < b1; ++b) dsum += S.dB[b];
     if (dsum > 0.0) val = sf::mul(sf::mul_pow2(D.mi[i], -1), rcp64(dsum));
   }
   block_min_to(val, &c.clk->tau_bits);
@@ -217,6 +206,55 @@ __global__ void __maxnreg__(48) k_tau(Src src, int sliced) {
   tau_body<DIM, MX, Src>(src, sliced);
 }
 
+// What a stage needs of boundary entry b, one thread per entry (the first threads of the edge sweep, so that
+// the sweeps over rows read it instead of working it out inside their rows: the powers, roots and
+// divisions of an entry are a chain of FP64 operations that held up its row's whole warp, in every sweep
+// again): the boundary state (Sec. 4.1), d_i^{d,k} = |c_i^{d,k}| lambda_max^+(U_i, U^{d,k}, n_i^k)
+// (Sec. 4.2, eq. (eq:dij_low_order_modified); interior state on the left), both fluxes times c_i^{d,k},
+// and rho and s~ of the boundary bar state (eq. (BoundaryBarState)).  At Q2 301 x 259 with open sides, in us per
+// launch: k_low 326 -> 213, k_tau 138 -> 34, k_high 414 -> 322, k_edge 241 -> 245.  A function of its own, so
+// that its registers are not the edges': inlined, the edges spill 136 bytes in place of 44.
+template <int DIM, bool MX>
+__device__ __noinline__ void boundary_entry(const Ctx& c, int b) {
+  constexpr int M = DIM + 2;
+  const Dev& D = c.D;
+  const Scratch& S = c.S;
+  const size_t n = D.n, nb = D.nb;
+  const int i = D.bnode[b];
+  const double* P = S.prim;
+  double Ui[M], nv[DIM], UB[M];
+  load_state<DIM>(c.U, D.n, i, Ui);
+  const double irho_i = P[PR_IRHO * n + i], p_i = P[PR_P * n + i];
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) nv[k] = D.bn[(size_t)k * nb + b];
+  boundary_state<DIM>(D, b, Ui, c.bdata, nv, UB);
+  const double irB = rcp64(UB[0]);
+  const double pB = sf::mul(D.gm1, fma(-sf::mul_pow2(dot<DIM>(UB + 1, UB + 1), -1), irB, UB[DIM + 1]));
+  const double mnL = dot<DIM>(Ui + 1, nv), mnR = dot<DIM>(UB + 1, nv);
+  const double uL = sf::mul(mnL, irho_i), uR = sf::mul(mnR, irB);
+  const double cnm = D.bnorm[b];
+  double ipB, aB, pmeB;
+  prim_of<MX>(D, UB[0], irB, pB, &ipB, &aB, &pmeB);
+  const double d = sf::mul(cnm, lambda_pair<MX>(D, uL, p_i, irho_i, P[PR_IP * n + i], P[PR_A * n + i],
+                                                P[PR_PME * n + i], uR, pB, irB, ipB, aB, pmeB));
+  S.dB[b] = d;
+  double fi[M], fB[M], Ub[M];
+  flux_n<DIM>(Ui, nv, mnL, uL, p_i, fi);
+  flux_n<DIM>(UB, nv, mnR, uR, pB, fB);
+  const double t = sf::mul(sf::mul_pow2(cnm, -1), rcp64(d));
+#pragma unroll
+  for (int q = 0; q < M; ++q) {
+    S.UB[q * nb + b] = UB[q];
+    S.gB[q * nb + b] = sf::mul(cnm, fB[q]);
+    S.gI[q * nb + b] = sf::mul(cnm, fi[q]);
+    Ub[q] = fma(-t, fB[q] - fi[q], sf::mul_pow2(Ui[q] + UB[q], -1));
+  }
+  double irb;
+  const double rg = rho_neg_gamma(D, Ub[0], &irb);
+  S.bbar[b] = Ub[0];
+  S.bbar[nb + b] = sf::mul(rg, fma(-sf::mul_pow2(dot<DIM>(Ub + 1, Ub + 1), -1), irb, Ub[DIM + 1]));
+}
+
 // Edge sweep, one thread per undirected stencil edge {i, j} (i < j): the quantities of a pair that are
 // symmetric in i and j are computed once and written to both entries (i, j) and (j, i):
 //  - d_ij^L = d_ji^L = |c_ij| lambda_max^+(U_i, U_j, n_ij) (Sec. 3.1, eq. (eq:dij_low_order); the bound
@@ -224,6 +262,7 @@ __global__ void __maxnreg__(48) k_tau(Src src, int sliced) {
 //  - the bar state Ubar_ij = Ubar_ji (eq. (UsualBarState)), of which only rho and s~ are kept (for the
 //    local bounds of eq. (eq:local_bounds));
 //  - G_ij = f(U_j) c_ij and G_ji = f(U_i) c_ji = -|c_ij| f(U_i) n_ij for the row sums of sweep A.
+// The first threads take the boundary entries.
 // The mixed path (MX) takes lambda from lambda_pair<true> and the entropy power of the bar state in FP32;
 // the fluxes, G and the bar state itself stay FP64.
 template <int DIM, bool MX, class Src>
@@ -235,8 +274,13 @@ __device__ __forceinline__ void edge_body(const Src& src) {
   if (finished(c)) return;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const int k = lb * blockDim.x + threadIdx.x;
-  if (k >= D.ne) return;
+  const unsigned slot = lb * blockDim.x + threadIdx.x, nbs = boundary_slots(D.nb);
+  if (slot < nbs) {
+    if (slot < (unsigned)D.nb) boundary_entry<DIM, MX>(c, (int)slot);
+    return;
+  }
+  const unsigned k = slot - nbs;
+  if (k >= (unsigned)D.ne) return;
   const size_t n = D.n, nnz = D.nnz;
   const int e = D.edge_e[k], i = D.edge_i[k];
   const int j = D.col[e], t = D.tr[e];
@@ -311,21 +355,20 @@ __device__ __forceinline__ void edge_body(const Src& src) {
 // sweep want resident warps to hide their latency (2.77 ms per launch at Q2 1024^2, against 3.04 with one
 // block of 512 at 82 registers).
 template <int DIM, bool MX, class Src>
-__global__ void __launch_bounds__(kThreads, 2) k_edge(Src src) {
+__global__ void __launch_bounds__(kThreads, 2) k_edge(const __grid_constant__ Src src) {
   edge_body<DIM, MX, Src>(src);
 }
 
 // Sweep A, one thread per row i, after the edge sweep:
-//  - the row sums of d_ij^L and f(U_j) c_ij from the edge sweep; boundary states and viscosities (Sec. 4.1;
-//    Sec. 4.2, eq. (eq:dij_low_order_modified));
+//  - the row sums of d_ij^L and f(U_j) c_ij and the boundary terms, all from the edge sweep;
 //  - the low-order update of Sec. 4.2, eq. (cijdijschememodified), and the CFL check (CFLcond);
 //  - the entropy-viscosity indicator N_i = R_i / D_i (Sec. 5.2);
 //  - the one-hop aggregates of the local bounds (Sec. 5.4, eq. (eq:local_bounds)): min/max of rho_j,
 //    rho(Ubar_jk), rho_k and min of s~ over node j's stencil, with the bar states of
-//    eq. (UsualBarState); and rho, s~ of node i's boundary bar states (eq. (BoundaryBarState)).
+//    eq. (UsualBarState).
 // With order LOW (or no limiter pass) it also writes U_out = alpha U_base + (1 - alpha) U^L.
-// The mixed path (MX) computes the indicator in FP32 (its sums from FP64 flux differences) and the
-// boundary wave-speed bounds with lambda_pair<true>; the low-order update stays FP64.
+// The mixed path (MX) computes the indicator in FP32 (its sums from FP64 flux differences); the low-order
+// update stays FP64.
 template <int DIM, bool MX, class Src>
 __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_out) {
   constexpr int M = DIM + 2;
@@ -343,8 +386,8 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
   const double* P = S.prim;
   double Ui[M];
   load_state<DIM>(U, D.n, i, Ui);
-  const double irho_i = P[PR_IRHO * n + i], p_i = P[PR_P * n + i], ip_i = P[PR_IP * n + i],
-               a_i = P[PR_A * n + i], pme_i = P[PR_PME * n + i], f_i = P[PR_F * n + i], st_i = P[PR_ST * n + i];
+  const double irho_i = P[PR_IRHO * n + i], ip_i = P[PR_IP * n + i], f_i = P[PR_F * n + i],
+               st_i = P[PR_ST * n + i];
   using Acc = std::conditional_t<MX, float, double>;  // arithmetic of the indicator's sums
   // RHS^L = sum_j f(U_j) c_ij - sum_j d_ij (U_j - U_i) + boundary terms, accumulated as its two sums
   // (sg, sdu); the indicator's Fsum reuses sg
@@ -391,38 +434,20 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
 #pragma unroll
     for (int q = 0; q < M; ++q) Fsum[q] += sg[q];
   }
-  for (int b = D.b_ptr[i]; b < D.b_ptr[i + 1]; ++b) {
-    double nv[DIM], UB[M];
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) nv[k] = D.bn[(size_t)k * D.nb + b];
-    boundary_state<DIM>(D, b, Ui, c.bdata, nv, UB);
-    double irB = 1.0 / UB[0];
-    double pB = sf::mul(D.gm1, internal_energy<DIM>(UB));
-    const double mnL = dot<DIM>(Ui + 1, nv), mnR = dot<DIM>(UB + 1, nv);
-    const double uL = sf::mul(mnL, irho_i), uR = sf::mul(mnR, irB);
-    double cnm = D.bnorm[b];
-    double ipB, aB, pmeB;
-    prim_of<MX>(D, UB[0], irB, pB, &ipB, &aB, &pmeB);
-    double d = sf::mul(cnm, lambda_pair<MX>(D, uL, p_i, irho_i, ip_i, a_i, pme_i, uR, pB, irB, ipB, aB, pmeB));
-    S.dB[b] = d;
+  for (int b = D.b_ptr[i], b1 = D.b_ptr[i + 1]; b < b1; ++b) {
+    const size_t nb = D.nb;
+    const double d = S.dB[b];
     dsum += d;
-    double fi[M], fB[M];
-    flux_n<DIM>(Ui, nv, mnL, uL, p_i, fi);
-    flux_n<DIM>(UB, nv, mnR, uR, pB, fB);
-    double t = cnm / sf::mul_pow2(d, 1);
-    double Ub[M];
 #pragma unroll
     for (int q = 0; q < M; ++q) {
-      sg[q] = fma(cnm, fB[q], sg[q]);
-      sdu[q] = fma(d, UB[q] - Ui[q], sdu[q]);
+      const double gi = S.gI[q * nb + b];
+      sg[q] += S.gB[q * nb + b];
+      sdu[q] = fma(d, S.UB[q * nb + b] - Ui[q], sdu[q]);
       if constexpr (MX)
-        Fsum[q] -= to_f32(cnm * fi[q]);
+        Fsum[q] -= to_f32(gi);
       else
-        Fsum[q] = fma(-cnm, fi[q], Fsum[q]);
-      Ub[q] = fma(-t, fB[q] - fi[q], 0.5 * (Ui[q] + UB[q]));
+        Fsum[q] -= gi;
     }
-    S.bbar[b] = Ub[0];
-    S.bbar[(size_t)D.nb + b] = sf::mul(pow(Ub[0], -D.gamma), internal_energy<DIM>(Ub));
   }
   const double inv_mi = D.inv_mi[i];
   if (sf::mul(sf::mul(sf::mul_pow2(tau, 1), dsum), inv_mi) > 1.0 + 1e-12) atomicOr(S.flags, (unsigned)GDG_FLAG_CFL);
