@@ -151,9 +151,10 @@ inline void set_eos(Dev& D, double gamma) {
 struct Scratch {
   double* prim;    // [NPRIM][n]
   double* dL;      // [nnz]
-  double* G;       // [m][nnz] f(U_j) c_ij of stencil entries (from the edge sweep)
+  double* G;       // [m][nnz] (f(U_j) - f(U_i)) c_ij of stencil entries (from the edge sweep; symmetric in i, j)
+  double* psi;     // [nnz] (m_j . c_ij)(f_j - f_i), the indicator's term of the entry (mixed: m_j . c_ij)
   double* barR;    // [nnz] rho of the bar state Ubar_ij (symmetric in i, j)
-  double* barS;    // [nnz] s~ of the bar state
+  double* barS;    // [nnz] the least s~ of U_i, U_j and the bar state (symmetric in i, j)
   double* dB;      // [nb]
   double* bbar;    // [2][nb] rho and s~ of the boundary bar states
   double* UB;      // [m][nb] boundary states U_i^{d,k}

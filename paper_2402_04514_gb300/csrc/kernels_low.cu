@@ -259,9 +259,14 @@ __device__ __noinline__ void boundary_entry(const Ctx& c, int b) {
 // symmetric in i and j are computed once and written to both entries (i, j) and (j, i):
 //  - d_ij^L = d_ji^L = |c_ij| lambda_max^+(U_i, U_j, n_ij) (Sec. 3.1, eq. (eq:dij_low_order); the bound
 //    is symmetric under (U_i, U_j, n) -> (U_j, U_i, -n), which is also what makes d^L symmetric);
-//  - the bar state Ubar_ij = Ubar_ji (eq. (UsualBarState)), of which only rho and s~ are kept (for the
-//    local bounds of eq. (eq:local_bounds));
-//  - G_ij = f(U_j) c_ij and G_ji = f(U_i) c_ji = -|c_ij| f(U_i) n_ij for the row sums of sweep A.
+//  - the bar state Ubar_ij = Ubar_ji (eq. (UsualBarState)), of which only rho is kept, and the least s~ of it
+//    and both nodes (for the local bounds of eq. (eq:local_bounds));
+//  - the flux difference G_ij = (f(U_j) - f(U_i)) c_ij = G_ji, whose row sums sweep A takes in place of those of
+//    f(U_j) c_ij (they differ by f(U_i) sum_j c_ij, which Lemma LemPart gives in boundary terms): one symmetric
+//    array where f(U_j) c_ij and f(U_i) c_ji were two, so that a row reads only its own entries.  With the
+//    indicator's entry term computed here too, sweep A's loop has 14 FP64 operations per entry in place of 19
+//    and 44 bytes less to read (2.49 -> 1.89 ms per launch at Q2 1024^2);
+//  - the indicator's term (m_j . c_ij)(f_j - f_i) of Sec. 5.2 for both rows.
 // The first threads take the boundary entries.
 // The mixed path (MX) takes lambda from lambda_pair<true> and the entropy power of the bar state in FP32;
 // the fluxes, G and the bar state itself stay FP64.
@@ -317,9 +322,18 @@ __device__ __forceinline__ void edge_body(const Src& src) {
   double W[M];
 #pragma unroll
   for (int q = 0; q < M; ++q) {
-    S.G[q * nnz + e] = gj[q];
-    S.G[q * nnz + t] = -gi[q];
-    W[q] = fma(-r, gj[q] - gi[q], Ui[q] + Uj[q]);
+    const double df = gj[q] - gi[q];
+    S.G[q * nnz + e] = df;
+    S.G[q * nnz + t] = df;
+    W[q] = fma(-r, df, Ui[q] + Uj[q]);
+  }
+  if constexpr (MX) {
+    S.psi[e] = gj[0];
+    S.psi[t] = -gi[0];
+  } else {
+    const double fd = P[PR_F * n + j] - P[PR_F * n + i];
+    S.psi[e] = sf::mul(gj[0], fd);
+    S.psi[t] = sf::mul(gi[0], fd);  // (-gi)(f_i - f_j)
   }
   double Ub[M];
   Ub[0] = sf::mul_pow2(W[0], -1);
@@ -347,6 +361,7 @@ __device__ __forceinline__ void edge_body(const Src& src) {
   }
   S.barR[e] = Ub[0];
   S.barR[t] = Ub[0];
+  stb = pmin(stb, pmin(P[PR_ST * n + i], P[PR_ST * n + j]));
   S.barS[e] = stb;
   S.barS[t] = stb;
 }
@@ -390,9 +405,9 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
                st_i = P[PR_ST * n + i];
   using Acc = std::conditional_t<MX, float, double>;  // arithmetic of the indicator's sums
   // RHS^L = sum_j f(U_j) c_ij - sum_j d_ij (U_j - U_i) + boundary terms, accumulated as its two sums
-  // (sg, sdu); the indicator's Fsum reuses sg
+  // (sg, sdu); the indicator's sum is sg
   double sg[M], sdu[M];
-  Acc Fsum[M];
+  Acc Fsum[M];  // (mixed only)
 #pragma unroll
   for (int q = 0; q < M; ++q) {
     sg[q] = sdu[q] = 0.0;
@@ -404,7 +419,7 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
   const size_t nnz = D.nnz;
   const int e1 = D.sten_end[i];
   for (int e = D.rbeg[i]; e < e1; e += kEll) {  // I(i)
-    const int j = D.col[e], t = D.tr[e];
+    const int j = D.col[e];
     const double d = S.dL[e];
     dsum += d;
     double Uj[M];
@@ -414,26 +429,22 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
       const double ge = S.G[q * nnz + e];
       sg[q] += ge;
       sdu[q] = fma(d, Uj[q] - Ui[q], sdu[q]);
-      // Fsum = sum_j (f(U_j) - f(U_i)) c_ij: here the f(U_i) c_ij terms, sg is added after the loop (the
-      // two sums are exact negatives of each other term by term on a stencil holding one state); the
-      // mixed path sums the FP64 differences in FP32
-      if constexpr (MX)
-        Fsum[q] += to_f32(ge + S.G[q * nnz + t]);
-      else
-        Fsum[q] += S.G[q * nnz + t];
+      if constexpr (MX) Fsum[q] += to_f32(ge);  // the mixed path sums the FP64 differences in FP32
     }
     if constexpr (MX)
-      psum += to_f32(S.G[e]) * (to_f32(P[PR_F * n + j]) - to_f32(f_i));
+      psum += to_f32(S.psi[e]) * (to_f32(P[PR_F * n + j]) - to_f32(f_i));
     else
-      psum = fma(S.G[e], P[PR_F * n + j] - f_i, psum);  // (m_j . c_ij) (f_j - f_i)
+      psum += S.psi[e];
     lo = pmin(lo, pmin(Uj[0], S.barR[e]));
     hi = pmax(hi, pmax(Uj[0], S.barR[e]));
-    sl = pmin(sl, pmin(P[PR_ST * n + j], S.barS[e]));
+    sl = pmin(sl, S.barS[e]);
   }
-  if constexpr (!MX) {
+  // sg is now the sum of (f(U_j) - f(U_i)) c_ij; with the boundary terms, Fsum = sg - f(U_i) sum_k c_i^{d,k} =
+  // sum_j f(U_j) c_ij and the right-hand side takes Fsum + sum_k f(U^{d,k}) c_i^{d,k}.  On a stencil that
+  // holds one state every term is zero, or cancels with its partner, exactly.
+  double sgB[M];
 #pragma unroll
-    for (int q = 0; q < M; ++q) Fsum[q] += sg[q];
-  }
+  for (int q = 0; q < M; ++q) sgB[q] = 0.0;
   for (int b = D.b_ptr[i], b1 = D.b_ptr[i + 1]; b < b1; ++b) {
     const size_t nb = D.nb;
     const double d = S.dB[b];
@@ -441,19 +452,17 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
 #pragma unroll
     for (int q = 0; q < M; ++q) {
       const double gi = S.gI[q * nb + b];
-      sg[q] += S.gB[q * nb + b];
+      sgB[q] += S.gB[q * nb + b];
+      sg[q] -= gi;
       sdu[q] = fma(d, S.UB[q * nb + b] - Ui[q], sdu[q]);
-      if constexpr (MX)
-        Fsum[q] -= to_f32(gi);
-      else
-        Fsum[q] -= gi;
+      if constexpr (MX) Fsum[q] -= to_f32(gi);
     }
   }
   const double inv_mi = D.inv_mi[i];
   if (sf::mul(sf::mul(sf::mul_pow2(tau, 1), dsum), inv_mi) > 1.0 + 1e-12) atomicOr(S.flags, (unsigned)GDG_FLAG_CFL);
   double rhs[M];
 #pragma unroll
-  for (int q = 0; q < M; ++q) rhs[q] = sg[q] - sdu[q];
+  for (int q = 0; q < M; ++q) rhs[q] = (sg[q] + sgB[q]) - sdu[q];
   double UL[M];
 #pragma unroll
   for (int q = 0; q < M; ++q) UL[q] = fma(-sf::mul(tau, inv_mi), rhs[q], Ui[q]);
@@ -513,8 +522,8 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
     double R = psum, Dn = fabs(psum);
 #pragma unroll
     for (int q = 0; q < M; ++q) {
-      R = fma(-grad[q], Fsum[q], R);
-      Dn = fma(fabs(grad[q]), fabs(Fsum[q]), Dn);
+      R = fma(-grad[q], sg[q], R);
+      Dn = fma(fabs(grad[q]), fabs(sg[q]), Dn);
     }
     S.N[i] = Dn > 0.0 ? sf::mul(R, rcp64(Dn)) : 0.0;
   }
