@@ -7,25 +7,19 @@
 #include <cstdint>
 
 #include "../../include/gdg.h"
-#include "softfp64.cuh"
+#include "fixfp64.cuh"
 
 namespace gdg {
 
 // Per-node primitive record written by k_prim and read for every neighbour in the sweeps.
 enum { PR_IRHO = 0, PR_P, PR_A, PR_PME, PR_F, PR_ST, PR_IP, NPRIM };
 
-// Constants of the Newton roots x^{-1/q} (rootinv, below).
+// Constants of the roots x^{-1/q} (rootinv, below).
 struct RootQ {
-  int q;
-  double iq, c2;  // 1 / q and (q + 1) / (2 q^2)
+  sf::rootc c;
+  double iq;  // 1 / q
 };
-__host__ __device__ inline RootQ root_q(int q) {
-  RootQ r;
-  r.q = q;
-  r.iq = 1.0 / q;
-  r.c2 = 0.5 * r.iq * (1.0 + r.iq);
-  return r;
-}
+__host__ __device__ inline RootQ root_q(int q) { return RootQ{sf::root_const(q), 1.0 / q}; }
 
 // Per-entry arrays are stored as sliced ELL.  The elements are taken in groups of kEll consecutive
 // elements; slice (g, l) holds the rows of local index l of the group's elements, entry k of the row of
@@ -138,7 +132,7 @@ inline void set_eos(Dev& D, double gamma) {
   D.ie_root = (D.ie > 0 && D.ie <= 16) ? D.ie : 0;
   D.root_gq = root_q(D.gq > 0 ? D.gq : 1);
   D.root_ie = root_q(D.ie_root > 0 ? D.ie_root : 1);
-  D.root_gpq = root_q(D.gq > 0 ? D.gp + D.gq : 1);
+  D.root_gpq = root_q(D.gq > 0 && D.gp + D.gq <= 16 ? D.gp + D.gq : 1);
   D.inv_gp1 = 1.0 / (gamma + 1.0);
   D.gamma_f = (float)gamma;
   D.gm1h_f = (float)(0.5 * D.gm1);
@@ -424,35 +418,6 @@ inline cudaError_t launch_one(int kern, int dim, const Ctx& c, int arg, const Sc
 // ------------------------------------------------------------------------------------------------
 // Device helpers (Euler equations of Sec. 2.2 and the pieces of Sec. 3-5 used by several kernels).
 
-// a * b on the integer pipe (Soft, csrc/softfp64.cuh) or on the FP64 pipe: the same bits either way.  The
-// deferred line searches take the FP64 pipe: their few active lanes per warp hide less of the integer
-// routine's latency than they gain from the freed FP64 slots (k_lsfix 0.37 -> 0.41 ms per launch at Q2
-// 1024^2 with the integer products).
-template <bool Soft>
-__device__ __forceinline__ double mulp(double a, double b) {
-  if constexpr (Soft)
-    return sf::mul(a, b);
-  else
-    return a * b;
-}
-
-// x^k for an integer k >= 0 by binary powering without a trailing square (k = 5, 7, 12 take 3, 4, 4
-// multiplications).
-template <bool Soft = true>
-__device__ __forceinline__ double ipow(double x, int k) {
-  if (k <= 0) return 1.0;
-  while (!(k & 1)) {
-    x = mulp<Soft>(x, x);
-    k >>= 1;
-  }
-  double r = x;
-  while (k >>= 1) {
-    x = mulp<Soft>(x, x);
-    if (k & 1) r = mulp<Soft>(r, x);
-  }
-  return r;
-}
-
 // FP64 -> FP32 by integer operations only (no instruction on the FP64 pipe, where the hardware conversion
 // costs about 1.6 FMA issue slots): exponent rebias and the significand truncated to 23 bits (relative
 // error < 2^-23) for values in the FP32 normal range, +-0 -> +-0.  Every other value (below the FP32
@@ -504,84 +469,50 @@ __device__ __forceinline__ double abs_bits(double x) {
 __device__ __forceinline__ bool is_zero_bits(double x) { return (__double_as_longlong(x) << 1) == 0; }
 __device__ __forceinline__ bool is_one_bits(double x) { return __double_as_longlong(x) == 0x3ff0000000000000LL; }
 
-// FP64 reciprocal from the FP32 reciprocal y0 of x in FP32 (relative error e = 1 - x y0 below 2^-22):
-// 1/x = y0 / (1 - e) = y0 (1 + e + e^2 + ...), summed through e^2 in one fused update, leaves
-// e^3 < 2^-66 plus the rounding of the last FMA, so the result is within 2 ulp of 1/x.  Costs 3 FP64
-// operations instead of a full FP64 division on a chip whose FP64 pipe is the bottleneck.  Arguments
-// outside the FP32 normal range take the IEEE division.
+// 1/x, sqrt(x) and x^{-1/q} (x > 0, 1 <= q <= 16) on the integer pipe (fixfp64.cuh), within 0.53 ulp; zeros,
+// infinities, NaN and the ends of the range take the FP64 operation, out of line.
+static __device__ __noinline__ __attribute__((const)) double rcp_hw(double x) { return 1.0 / x; }
+static __device__ __noinline__ __attribute__((const)) double sqrt_hw(double x) { return sqrt(x); }
+static __device__ __noinline__ __attribute__((const)) double pow_hw(double x, double y) { return pow(x, y); }
+static __device__ __noinline__ __attribute__((const)) double ratio_pow_hw(double x, double y, double p) { return pow(x / y, p); }
 __device__ __forceinline__ double rcp64(double x) {
-  float xf = d2f_fast(x);
-  float ax = fabsf(xf);
-  if (!(ax > 1e-37f && ax < 1e37f)) return 1.0 / x;
-  const double y = f2d_fast(__frcp_rn(xf));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  if (__builtin_expect(!sf::rcp_ok(x), 0)) return rcp_hw(x);
+  return sf::rcp(x);
 }
-
-// sqrt(x) for x in the FP32 normal range by two Heron corrections s <- s + (x - s^2) h from s0 = x y0,
-// with y0 the FP32 reciprocal square root (relative error below 2^-21) and h = y0 / 2 held fixed: each
-// correction multiplies the relative error by about that of h and adds half its square
-// (2^-21 -> 2^-41 -> 2^-61), so the result is within an ulp or so of sqrt(x).  5 FP64 operations instead of
-// CUDA's square root with its special-case handling.  Other arguments take sqrt.
 __device__ __forceinline__ double sqrt64(double x) {
-  const float xf = d2f_fast(x);
-  if (!(xf > 1e-37f && xf < 1e37f)) return sqrt(x);
-  const float yf = rsqrtf(xf);
-  const double h = f2d_fast(0.5f * yf);
-  double s = sf::mul(x, f2d_fast(yf));
-  s = fma(fma(-s, s, x), h, s);
-  return fma(fma(-s, s, x), h, s);
+  if (__builtin_expect(!sf::pos_normal(x), 0)) return sqrt_hw(x);
+  return sf::sqrt_pos(x);
 }
-
-// y = x^{-1/q} for x > 0 and 1 <= q <= 16.  From the FP32 seed y0 = exp2(-log2(x) / q), with
-// t = 1 - x y0^q and x^{-1/q} = y0 (1 - t)^{-1/q}, one step y0 (1 + t/q + (q+1)/(2q^2) t^2) sums the
-// binomial series through t^2; the rest, |binom(-1/q, 3)| |t|^3 (1 + O(t)) with |binom(-1/q, 3)| <= 1
-// (0.09 for q >= 5), is below 2^-56 when |t| <= 2^-19, which the seed's 2^-22 relative error (times q)
-// gives for arguments near 1.  Far
-// from 1 log2f's absolute error grows with |log2 x| and the seed can be worse; then one Newton step
-// y <- y + y (1 - x y^q) / q squares the remaining error.  Arguments outside the FP32 normal range use pow.
-template <bool Soft = true>
 __device__ __forceinline__ double rootinv(double x, const RootQ& r) {
-  float xf = d2f_fast(x);
-  if (!(xf > 1e-37f && xf < 1e37f)) return pow(x, -r.iq);
-  double y = f2d_fast(exp2f(-log2f(xf) / (float)r.q));
-  const double t = fma(-x, ipow<Soft>(y, r.q), 1.0);
-  y = fma(mulp<Soft>(y, t), fma(r.c2, t, r.iq), y);
-  // |t| > 2^-19, compared on the bit patterns (integer pipe)
-  if ((__double_as_longlong(t) & 0x7fffffffffffffffLL) > 0x3ec0000000000000LL) {
-    const double t2 = fma(-x, ipow<Soft>(y, r.q), 1.0);
-    y = fma(y * t2, r.iq, y);
-  }
-  return y;
+  if (__builtin_expect(!sf::pos_normal(x), 0)) return pow_hw(x, -r.iq);
+  return sf::uf_dbl(sf::uf_rootinv(x, r.c));
 }
 
 // rho^{-gamma} and 1/rho together.  With gamma = p/q (p > q): y = rho^{-1/q}, 1/rho = y^q and
-// rho^{-gamma} = y^p, as y^q y^{p-q} (Share: fewer multiplications, one longer chain; faster in the edge
-// sweep) or by its own powering (measured faster in k_prim).
-template <bool Share = true>
+// rho^{-gamma} = y^q y^{p-q}, unpacked until the end.
 __device__ __forceinline__ double rho_neg_gamma(const Dev& D, double rho, double* inv_rho) {
-  if (D.gq > 0) {
-    const double y = rootinv(rho, D.root_gq);
-    const double yq = ipow(y, D.gq);
-    *inv_rho = yq;
-    return Share ? sf::mul(yq, ipow(y, D.gp - D.gq)) : ipow(y, D.gp);
+  if (D.gq > 0 && sf::pos_normal(rho)) {
+    const sf::uf y = sf::uf_rootinv(rho, D.root_gq.c);
+    const sf::uf yq = sf::uf_pow(y, D.gq);
+    *inv_rho = sf::uf_dbl(yq);
+    return sf::uf_dbl(sf::uf_mul(yq, sf::uf_pow(y, D.gp - D.gq)));
   }
   *inv_rho = rcp64(rho);
-  return pow(rho, -D.gamma);
+  return pow_hw(rho, -D.gamma);
 }
 
 // rho^gamma and 1/rho together.  With gamma = p/q, k = ceil(p/q) and c = kq - p (0 <= c < q):
-// rho^gamma = rho^k y^c and 1/rho = y^q = y^c y^{q-c}.
-template <bool Soft = true>
+// rho^gamma = rho^k y^c and 1/rho = y^q, y = rho^{-1/q}.
 __device__ __forceinline__ double rho_pow_gamma(const Dev& D, double rho, double* inv_rho) {
-  if (D.gq > 0) {
-    const double y = rootinv<Soft>(rho, D.root_gq);
-    const double yc = ipow<Soft>(y, D.gc);
-    *inv_rho = mulp<Soft>(yc, ipow<Soft>(y, D.gq - D.gc));
-    return mulp<Soft>(ipow<Soft>(rho, D.gk), yc);
+  if (D.gq > 0 && sf::pos_normal(rho)) {
+    const sf::uf y = sf::uf_rootinv(rho, D.root_gq.c);
+    sf::uf r = sf::uf_pow(sf::uf_of(rho), D.gk);
+    if (D.gc > 0) r = sf::uf_mul(r, sf::uf_pow(y, D.gc));
+    *inv_rho = sf::uf_dbl(sf::uf_pow(y, D.gq));
+    return sf::uf_dbl(r);
   }
   *inv_rho = rcp64(rho);
-  return pow(rho, D.gamma);
+  return pow_hw(rho, D.gamma);
 }
 
 // min / max of positive doubles through their bit patterns (IEEE order of positive numbers is the
@@ -606,8 +537,12 @@ __device__ __forceinline__ double lambda_max(const Dev& D, double uL, double pL,
   // (a positive double is a positive int64)
   auto pos = [](double x) { return __double_as_longlong(x) > 0 ? x : 0.0; };
   double num = pos(fma(-D.gm1h, uR - uL, aL + aR));
-  double r = sf::mul(num, rcp64(fma(aL, pmeL, sf::mul(aR, pmeR))));
-  double pt = D.ie > 0 ? ipow(r, D.ie) : pow(r, D.inv_e);
+  const double den = fma(aL, pmeL, sf::mul(aR, pmeR));
+  double pt;  // (num / den)^{1/e}
+  if (D.ie > 0 && sf::pos_normal(num) && sf::pos_normal(den))
+    pt = sf::uf_dbl(sf::uf_pow(sf::uf_mul(sf::uf_of(num), sf::uf_rcp(den)), D.ie));
+  else
+    pt = ratio_pow_hw(num, den, D.inv_e);
   double xL = pt - pL, xR = pt - pR;
   double sL = __double_as_longlong(xL) > 0 ? sqrt64(fma(sf::mul(D.k13, xL), ipL, 1.0)) : 1.0;
   double sR = __double_as_longlong(xR) > 0 ? sqrt64(fma(sf::mul(D.k13, xR), ipR, 1.0)) : 1.0;
@@ -712,7 +647,7 @@ __device__ __forceinline__ float lambda_max_mx(const Dev& D, float uL, float pL,
 __device__ __forceinline__ void prim_fp64(const Dev& D, double irho, double p, double* ip, double* a, double* pme) {
   *ip = rcp64(p);
   *a = sqrt64(sf::mul(sf::mul(D.gamma, p), irho));
-  *pme = D.ie_root > 0 ? rootinv(p, D.root_ie) : pow(p, -D.e_exp);
+  *pme = D.ie_root > 0 ? rootinv(p, D.root_ie) : pow_hw(p, -D.e_exp);
 }
 
 // 1/p, a and p^{-e} of a state that k_prim does not see (a boundary state), as each path computes them.
@@ -767,7 +702,8 @@ __device__ __forceinline__ double dot(const double* a, const double* b) {
   return s;
 }
 
-// The same on the FP64 pipe, for the line searches (mulp).
+// The same on the FP64 pipe, for the line searches: their few active lanes per warp hide less of the integer
+// product's latency than they gain from the freed FP64 slots.
 template <int DIM>
 __device__ __forceinline__ double dot_fp64(const double* a, const double* b) {
   double s = __dmul_rn(a[0], b[0]);
@@ -921,7 +857,7 @@ __device__ __forceinline__ double ls_psi(const Dev& D, const double* U0, const d
   if (!(V[0] > 0.0)) return -1.0;
   const double m2 = dot_fp64<DIM>(V + 1, V + 1);
   double irho;
-  double rg = rho_pow_gamma<false>(D, V[0], &irho);
+  double rg = rho_pow_gamma(D, V[0], &irho);
   return fma(-smin, rg, fma(-sf::mul_pow2(m2, -1), irho, V[DIM + 1]));
 }
 
@@ -934,7 +870,7 @@ __device__ __forceinline__ double ls_psi_dpsi(const Dev& D, const double* U0, co
   for (int q = 0; q < DIM + 2; ++q) V[q] = fma(s, A[q], U0[q]);
   const double mA = dot_fp64<DIM>(V + 1, A + 1), m2 = dot_fp64<DIM>(V + 1, V + 1);
   double irho;
-  double rg = rho_pow_gamma<false>(D, V[0], &irho);
+  double rg = rho_pow_gamma(D, V[0], &irho);
   // A_E - mA / rho + (A_rho / rho) (|m|^2 / (2 rho) - gamma s_min rho^gamma)
   *dpsi = fma(__dmul_rn(A[0], irho), fma(sf::mul_pow2(m2, -1), irho, -__dmul_rn(__dmul_rn(smin, D.gamma), rg)),
               fma(-mA, irho, A[DIM + 1]));

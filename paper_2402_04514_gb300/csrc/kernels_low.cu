@@ -75,16 +75,17 @@ __device__ __forceinline__ void prim_body(const Src& src) {
     return;
   }
   double ir;
-  double st = sf::mul(rho_neg_gamma<false>(D, Ui[0], &ir), eps);
+  double st = sf::mul(rho_neg_gamma(D, Ui[0], &ir), eps);
   P[PR_IRHO * n + i] = irho;
   P[PR_P * n + i] = p;
   P[PR_IP * n + i] = rcp64(p);
   P[PR_A * n + i] = sqrt64(sf::mul(sf::mul(D.gamma, p), irho));
-  P[PR_PME * n + i] = D.ie_root > 0 ? rootinv(p, D.root_ie) : pow(p, -D.e_exp);
+  P[PR_PME * n + i] = D.ie_root > 0 ? rootinv(p, D.root_ie) : pow_hw(p, -D.e_exp);
   // f = (gm1 s~)^{1/(gamma+1)} = x^{q/(p+q)} = x (x^{-1/(p+q)})^p for gamma = p/q
   double x = sf::mul(D.gm1, st);
-  P[PR_F * n + i] =
-      (D.gq > 0 && D.gp + D.gq <= 16) ? sf::mul(x, ipow(rootinv(x, D.root_gpq), D.gp)) : pow(x, D.inv_gp1);
+  P[PR_F * n + i] = (D.gq > 0 && D.gp + D.gq <= 16 && sf::pos_normal(x))
+                        ? sf::uf_dbl(sf::uf_mul(sf::uf_of(x), sf::uf_pow(sf::uf_rootinv(x, D.root_gpq.c), D.gp)))
+                        : pow_hw(x, D.inv_gp1);
   P[PR_ST * n + i] = st;
 }
 
@@ -367,8 +368,7 @@ __device__ __forceinline__ void edge_body(const Src& src) {
 }
 
 // Two 512-thread blocks per SM (64 registers, a few bytes of spills): the integer-pipe products of the
-// sweep want resident warps to hide their latency (2.77 ms per launch at Q2 1024^2, against 3.04 with one
-// block of 512 at 82 registers).
+// sweep want resident warps to hide their latency (2.18 ms per launch at Q2 1024^2).
 template <int DIM, bool MX, class Src>
 __global__ void __launch_bounds__(kThreads, 2) k_edge(const __grid_constant__ Src src) {
   edge_body<DIM, MX, Src>(src);
