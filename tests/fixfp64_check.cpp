@@ -39,7 +39,10 @@ int main(int argc, char** argv) {
     sq = fmaxl(sq, ulps(sf::sqrt_pos(x), sqrtl(X)));
     const int q = 1 + (int)(k % 16);
     const sf::uf y = sf::uf_rootinv(x, sf::root_const(q));
-    const long double ref = powl(X, -1.0L / q);
+    // powl rounds 1 / q, which far from 1 costs up to 2^-55 of the value: one Newton step on x r^q = 1 repairs it
+    long double ref = powl(X, -1.0L / q), prod = X;
+    for (int f = 0; f < q; ++f) prod *= ref;
+    ref += ref * (1.0L - prod) / q;
     if (!(y.m >> 63)) return printf("not normalised: %a q %d\n", x, q), 1;
     uroot = fmaxl(uroot, fabsl(value(y) / ref - 1.0L));
     root = fmaxl(root, ulps(sf::uf_dbl(y), ref));
