@@ -688,6 +688,11 @@ int gdg_max_dt(gdg_handle* h, const double* U, const double* bdata, double cfl, 
   if ((e = timed(h, GDG_K_MAXDT, s, [&] { return gdg::launch_one(gdg::KN_MAXDT, h->dim, c, 0, h->sched, s); })) !=
       cudaSuccess)
     return cuda_fail(e);
+  gdg::Sched sc = h->sched;  // the row sums take the launch shape and row order of this call's knobs
+  sc.bt[gdg::KN_TAU] = sc.bt[gdg::KN_MAXDT];
+  sc.slices = (sc.slices & ~(1 << gdg::KN_TAU)) | (((sc.slices >> gdg::KN_MAXDT) & 1) << gdg::KN_TAU);
+  if ((e = timed(h, GDG_K_TAU, s, [&] { return gdg::launch_one(gdg::KN_TAU, h->dim, c, 0, sc, s); })) != cudaSuccess)
+    return cuda_fail(e);
   unsigned long long bits = 0;
   if ((e = cudaMemcpyAsync(&bits, h->S.tau_bits, sizeof(bits), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
     return cuda_fail(e);

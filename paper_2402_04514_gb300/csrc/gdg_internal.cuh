@@ -349,6 +349,7 @@ __host__ __device__ inline int high_threads(int n_loc, int eb) { return (eb * n_
 __host__ __device__ inline unsigned boundary_slots(int nb) { return ((unsigned)nb + 31u) & ~31u; }
 inline long long kernel_blocks(int k, const Dev& D, const Sched& sc) {
   switch (k) {
+    case KN_MAXDT:
     case KN_EDGE: return ((long long)boundary_slots(D.nb) + D.ne + sc.bt[k] - 1) / sc.bt[k];
     case KN_HIGH: {  // the groups of kEll elements, each in kEll / eb blocks
       const int eb = high_elems_per_block(D.n_loc, sc.high_cap);

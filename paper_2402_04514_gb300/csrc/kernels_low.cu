@@ -128,11 +128,13 @@ __device__ __forceinline__ void block_min_to(double val, unsigned long long* dst
   }
 }
 
-// Sum over the row of d_ij^L plus the boundary viscosities, i.e. -d_ii of
-// eq. (eq:dij_low_order_supplement), then min over nodes of m_i / (2 |d_ii|), with d_ij^L evaluated here
-// (gdg_max_dt, before any stage).
+// d_ij^L of every stencil edge and d_i^{d,k} of every boundary entry (gdg_max_dt, before any stage), one thread
+// per boundary entry and then one per undirected edge as in the edge sweep below, stored for the row sums of k_tau
+// in arrays that the next stage overwrites before it reads them.  By edges each bound is worked out once
+// where a loop over rows does it twice, and no boundary row holds up its warp: 23 -> 8 us per call with
+// the row sums at Q2 33 x 47.
 template <int DIM, bool MX, class Src>
-__device__ __forceinline__ void maxdt_body(const Src& src, int sliced) {
+__device__ __forceinline__ void maxdt_body(const Src& src) {
   constexpr int M = DIM + 2;
   __shared__ Ctx sctx;
   int lb;
@@ -140,47 +142,46 @@ __device__ __forceinline__ void maxdt_body(const Src& src, int sliced) {
   if (finished(c)) return;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const double* U = c.U;
-  const int i = row_node(D, lb * blockDim.x + threadIdx.x, sliced);
-  double val = INFINITY;
-  if (i >= 0) {
-    size_t n = D.n;
+  const double* P = S.prim;
+  const size_t n = D.n, nnz = D.nnz;
+  const unsigned slot = lb * blockDim.x + threadIdx.x, nbs = boundary_slots(D.nb);
+  if (slot < nbs) {
+    if (slot >= (unsigned)D.nb) return;
+    const int i = D.bnode[slot];
     double Ui[M];
-    load_state<DIM>(U, D.n, i, Ui);
-    const double* P = S.prim;
-    double irho_i = P[PR_IRHO * n + i], p_i = P[PR_P * n + i], ip_i = P[PR_IP * n + i], a_i = P[PR_A * n + i],
-           pme_i = P[PR_PME * n + i];
-    double dsum = 0.0;
-    const int e1 = D.sten_end[i];
-    for (int e = D.rbeg[i]; e < e1; e += kEll) {  // I(i)
-      double cnm = D.cnorm[e];
-      int j = D.col[e];
-      double nv[DIM], mj[DIM];
-#pragma unroll
-      for (int k = 0; k < DIM; ++k) {
-        nv[k] = D.cn[(size_t)k * D.nnz + e];
-        mj[k] = U[(size_t)(1 + k) * n + j];
-      }
-      const double irho_j = P[PR_IRHO * n + j];
-      const double uL = sf::mul(dot<DIM>(Ui + 1, nv), irho_i), uR = sf::mul(dot<DIM>(mj, nv), irho_j);
-      dsum = fma(cnm, lambda_pair<MX>(D, uL, p_i, irho_i, ip_i, a_i, pme_i, uR, P[PR_P * n + j], irho_j,
-                                      P[PR_IP * n + j], P[PR_A * n + j], P[PR_PME * n + j]), dsum);
-    }
-    for (int b = D.b_ptr[i]; b < D.b_ptr[i + 1]; ++b)
-      dsum += boundary_viscosity<DIM, MX>(D, b, Ui, c.bdata, irho_i, p_i, ip_i, a_i, pme_i);
-    if (dsum > 0.0) val = sf::mul(sf::mul_pow2(D.mi[i], -1), rcp64(dsum));
+    load_state<DIM>(c.U, D.n, i, Ui);
+    S.bbar[slot] = boundary_viscosity<DIM, MX>(D, (int)slot, Ui, c.bdata, P[PR_IRHO * n + i], P[PR_P * n + i],
+                                               P[PR_IP * n + i], P[PR_A * n + i], P[PR_PME * n + i]);
+    return;
   }
-  block_min_to(val, S.tau_bits);
+  const unsigned k = slot - nbs;
+  if (k >= (unsigned)D.ne) return;
+  const int e = D.edge_e[k], i = D.edge_i[k], j = D.col[e];
+  double nv[DIM], mi[DIM], mj[DIM];
+#pragma unroll
+  for (int q = 0; q < DIM; ++q) {
+    nv[q] = D.cn[q * nnz + e];
+    mi[q] = c.U[(1 + q) * n + i];
+    mj[q] = c.U[(1 + q) * n + j];
+  }
+  const double ir_i = P[PR_IRHO * n + i], ir_j = P[PR_IRHO * n + j];
+  const double uL = sf::mul(dot<DIM>(mi, nv), ir_i), uR = sf::mul(dot<DIM>(mj, nv), ir_j);
+  const double d = sf::mul(D.cnorm[e], lambda_pair<MX>(D, uL, P[PR_P * n + i], ir_i, P[PR_IP * n + i], P[PR_A * n + i],
+                                                       P[PR_PME * n + i], uR, P[PR_P * n + j], ir_j, P[PR_IP * n + j],
+                                                       P[PR_A * n + j], P[PR_PME * n + j]));
+  S.barR[e] = d;
+  S.barR[D.tr[e]] = d;
 }
 
 template <int DIM, bool MX, class Src>
-__global__ void __launch_bounds__(kThreads) k_maxdt(Src src, int sliced) {
-  maxdt_body<DIM, MX, Src>(src, sliced);
+__global__ void __launch_bounds__(kThreads) k_maxdt(Src src) {
+  maxdt_body<DIM, MX, Src>(src);
 }
 
-// The same bound inside the fused SSP-RK3 step, after the edge sweep of the step's first stage: the row
-// sums of the stored d_ij^L and boundary viscosities, reduced into the instance's clock.  Capped at
-// 48 registers: the row sum is latency-bound and wants many warps.
+// Sums over the rows of d_ij^L plus the boundary viscosities, i.e. -d_ii of eq. (eq:dij_low_order_supplement), then
+// min over nodes of m_i / (2 |d_ii|): inside a fused step (with a clock) from what the edge sweep of its first
+// stage stored, into the clock; for gdg_max_dt from what k_maxdt stored.  Capped at 48 registers: the row
+// sum is latency-bound and wants many warps.
 template <int DIM, bool MX, class Src>
 __device__ __forceinline__ void tau_body(const Src& src, int sliced) {
   __shared__ Ctx sctx;
@@ -190,16 +191,18 @@ __device__ __forceinline__ void tau_body(const Src& src, int sliced) {
   const Dev& D = c.D;
   const Scratch& S = c.S;
   const int i = row_node(D, lb * blockDim.x + threadIdx.x, sliced);
+  const double* dL = c.clk ? S.dL : S.barR;
+  const double* dB = c.clk ? S.dB : S.bbar;
   double val = INFINITY;
   if (i >= 0) {
     double dsum = 0.0;
     const int e0 = D.rbeg[i], e1 = D.sten_end[i];
 #pragma unroll 4
-    for (int e = e0; e < e1; e += kEll) dsum += __ldg(S.dL + e);  // loads issued ahead of the in-order sum
-    for (int b = D.b_ptr[i], b1 = D.b_ptr[i + 1]; b < b1; ++b) dsum += S.dB[b];
+    for (int e = e0; e < e1; e += kEll) dsum += __ldg(dL + e);  // loads issued ahead of the in-order sum
+    for (int b = D.b_ptr[i], b1 = D.b_ptr[i + 1]; b < b1; ++b) dsum += dB[b];
     if (dsum > 0.0) val = sf::mul(sf::mul_pow2(D.mi[i], -1), rcp64(dsum));
   }
-  block_min_to(val, &c.clk->tau_bits);
+  block_min_to(val, c.clk ? &c.clk->tau_bits : S.tau_bits);
 }
 
 template <int DIM, bool MX, class Src>
@@ -541,7 +544,7 @@ cudaError_t low_launch(int kern, const Src& src, long long blocks, int threads, 
   const unsigned g = (unsigned)blocks;
   switch (kern) {
     case KN_PRIM: k_prim<DIM, MX, Src><<<g, threads, 0, s>>>(src); break;
-    case KN_MAXDT: k_maxdt<DIM, MX, Src><<<g, threads, 0, s>>>(src, sliced); break;
+    case KN_MAXDT: k_maxdt<DIM, MX, Src><<<g, threads, 0, s>>>(src); break;
     case KN_TAU: k_tau<DIM, MX, Src><<<g, threads, 0, s>>>(src, sliced); break;
     case KN_EDGE: k_edge<DIM, MX, Src><<<g, threads, 0, s>>>(src); break;
     case KN_LOW: k_low<DIM, MX, Src><<<g, threads, 0, s>>>(src, sliced, arg); break;
