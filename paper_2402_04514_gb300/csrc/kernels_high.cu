@@ -288,10 +288,12 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
 // 3.37 ms at 72, at 1024^2 Q2; with the integer-pipe products the FP64 path 4.36 ms at 64, 4.15 at 72).
 template <int DIM, class Src>
 __global__ void __maxnreg__(72) k_high(Src src, int eb) {
+  chain_begin();
   high_sweep<DIM, false, Src>(src, eb);
 }
 template <int DIM, class Src>
 __global__ void __maxnreg__(72) k_high_mixed(Src src, int eb) {
+  chain_begin();
   high_sweep<DIM, true, Src>(src, eb);
 }
 
@@ -304,10 +306,9 @@ cudaError_t high_launch(const Src& src, long long blocks, int n_loc, int eb, cud
     return cudaErrorInvalidValue;
   const int threads = high_threads(n_loc, eb);
   if constexpr (MX)
-    k_high_mixed<DIM, Src><<<(unsigned)blocks, threads, 0, s>>>(src, eb);
+    return launch_chained(k_high_mixed<DIM, Src>, (unsigned)blocks, threads, s, src, eb);
   else
-    k_high<DIM, Src><<<(unsigned)blocks, threads, 0, s>>>(src, eb);
-  return cudaGetLastError();
+    return launch_chained(k_high<DIM, Src>, (unsigned)blocks, threads, s, src, eb);
 }
 
 template <class Src>

@@ -90,6 +90,7 @@ __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last
 
 template <int DIM, class Src>
 __global__ void __maxnreg__(72) k_limit2(Src src, int sliced, int last) {
+  chain_begin();
   limit2_body<DIM, Src>(src, sliced, last);
 }
 
@@ -131,6 +132,7 @@ __device__ __forceinline__ void lsfix_body(const Src& src, int pass) {
 
 template <int DIM, class Src>
 __global__ void __launch_bounds__(kLsfixThreads) k_lsfix(Src src, int pass) {
+  chain_begin();
   lsfix_body<DIM, Src>(src, pass);
 }
 
@@ -180,6 +182,7 @@ __device__ __forceinline__ void final_body(const Src& src, int sliced) {
 
 template <int DIM, class Src>
 __global__ void __launch_bounds__(kLimThreads) k_final(Src src, int sliced) {
+  chain_begin();
   final_body<DIM, Src>(src, sliced);
 }
 
@@ -202,10 +205,12 @@ __device__ __forceinline__ void clock_advance(Clock* k, double dt_factor) {
 }
 
 __global__ void k_clock_one(Clock* k, double dt_factor) {
+  chain_begin();
   if (threadIdx.x == 0 && blockIdx.x == 0) clock_advance(k, dt_factor);
 }
 
 __global__ void k_clock_many(const Ctx* ctx, int ninst) {
+  chain_begin();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < ninst) clock_advance(ctx[k].clk, ctx[k].dt_factor);
 }
@@ -232,6 +237,7 @@ __device__ __forceinline__ void axpy_body(const Src& src) {
 
 template <int DIM, class Src>
 __global__ void __launch_bounds__(kLimThreads) k_axpy(Src src) {
+  chain_begin();
   axpy_body<DIM, Src>(src);
 }
 
@@ -242,13 +248,12 @@ cudaError_t limit_launch(int kern, const Src& src, long long blocks, int threads
   if (threads < 32 || threads > kLimThreads || threads % 32) return cudaErrorInvalidValue;
   const unsigned g = (unsigned)blocks;
   switch (kern) {
-    case KN_LIMIT2: k_limit2<DIM, Src><<<g, threads, 0, s>>>(src, sliced, arg); break;
-    case KN_FINAL: k_final<DIM, Src><<<g, threads, 0, s>>>(src, sliced); break;
-    case KN_AXPY: k_axpy<DIM, Src><<<g, threads, 0, s>>>(src); break;
-    case KN_LSFIX: k_lsfix<DIM, Src><<<g, kLsfixThreads, 0, s>>>(src, arg); break;
+    case KN_LIMIT2: return launch_chained(k_limit2<DIM, Src>, g, threads, s, src, sliced, arg);
+    case KN_FINAL: return launch_chained(k_final<DIM, Src>, g, threads, s, src, sliced);
+    case KN_AXPY: return launch_chained(k_axpy<DIM, Src>, g, threads, s, src);
+    case KN_LSFIX: return launch_chained(k_lsfix<DIM, Src>, g, kLsfixThreads, s, src, arg);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -276,14 +281,12 @@ cudaError_t launch_limit_file_many(int kern, int dim, const Many& m, long long b
 }
 
 cudaError_t launch_clock_one(Clock* clk, double dt_factor, cudaStream_t s) {
-  k_clock_one<<<1, 32, 0, s>>>(clk, dt_factor);
-  return cudaGetLastError();
+  return launch_chained(k_clock_one, 1u, 32, s, clk, dt_factor);
 }
 
 cudaError_t launch_clock_many(const Ctx* ctx, int ninst, cudaStream_t s) {
   if (ninst <= 0) return cudaSuccess;
-  k_clock_many<<<(ninst + 127) / 128, 128, 0, s>>>(ctx, ninst);
-  return cudaGetLastError();
+  return launch_chained(k_clock_many, (unsigned)(ninst + 127) / 128, 128, s, ctx, ninst);
 }
 
 #endif  // GDG_BODIES_ONLY

@@ -91,6 +91,7 @@ __device__ __forceinline__ void prim_body(const Src& src) {
 
 template <int DIM, bool MX, class Src>
 __global__ void __launch_bounds__(kThreads) k_prim(Src src) {
+  chain_begin();
   prim_body<DIM, MX, Src>(src);
 }
 
@@ -175,6 +176,7 @@ __device__ __forceinline__ void maxdt_body(const Src& src) {
 
 template <int DIM, bool MX, class Src>
 __global__ void __launch_bounds__(kThreads) k_maxdt(Src src) {
+  chain_begin();
   maxdt_body<DIM, MX, Src>(src);
 }
 
@@ -207,6 +209,7 @@ __device__ __forceinline__ void tau_body(const Src& src, int sliced) {
 
 template <int DIM, bool MX, class Src>
 __global__ void __maxnreg__(48) k_tau(Src src, int sliced) {
+  chain_begin();
   tau_body<DIM, MX, Src>(src, sliced);
 }
 
@@ -374,6 +377,7 @@ __device__ __forceinline__ void edge_body(const Src& src) {
 // sweep want resident warps to hide their latency (2.18 ms per launch at Q2 1024^2).
 template <int DIM, bool MX, class Src>
 __global__ void __launch_bounds__(kThreads, 2) k_edge(const __grid_constant__ Src src) {
+  chain_begin();
   edge_body<DIM, MX, Src>(src);
 }
 
@@ -534,6 +538,7 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
 
 template <int DIM, bool MX, class Src>
 __global__ void __launch_bounds__(kThreads) k_low(Src src, int sliced, int write_out) {
+  chain_begin();
   low_body<DIM, MX, Src>(src, sliced, write_out);
 }
 
@@ -543,14 +548,13 @@ cudaError_t low_launch(int kern, const Src& src, long long blocks, int threads, 
   if (threads < 32 || threads > kThreads || threads % 32) return cudaErrorInvalidValue;
   const unsigned g = (unsigned)blocks;
   switch (kern) {
-    case KN_PRIM: k_prim<DIM, MX, Src><<<g, threads, 0, s>>>(src); break;
-    case KN_MAXDT: k_maxdt<DIM, MX, Src><<<g, threads, 0, s>>>(src); break;
-    case KN_TAU: k_tau<DIM, MX, Src><<<g, threads, 0, s>>>(src, sliced); break;
-    case KN_EDGE: k_edge<DIM, MX, Src><<<g, threads, 0, s>>>(src); break;
-    case KN_LOW: k_low<DIM, MX, Src><<<g, threads, 0, s>>>(src, sliced, arg); break;
+    case KN_PRIM: return launch_chained(k_prim<DIM, MX, Src>, g, threads, s, src);
+    case KN_MAXDT: return launch_chained(k_maxdt<DIM, MX, Src>, g, threads, s, src);
+    case KN_TAU: return launch_chained(k_tau<DIM, MX, Src>, g, threads, s, src, sliced);
+    case KN_EDGE: return launch_chained(k_edge<DIM, MX, Src>, g, threads, s, src);
+    case KN_LOW: return launch_chained(k_low<DIM, MX, Src>, g, threads, s, src, sliced, arg);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <class Src>
