@@ -28,7 +28,8 @@ def _case(name):
 def test_factors_against_oracle(name):
     """l of both passes after seven stages.  Where the search iterates, its end is the root of psi to the tolerance 1e-14
     plus what psi's own rounding leaves open: a few ulp of E over |psi'| in row i or row j (l is their minimum); 16 ulp cover
-    both evaluations."""
+    both evaluations.  The second factor also moves with the first ones, each known to its own tolerance t: by l2 t / (1 - l1)
+    through the entry's remainder, and through the row's U^(1) by the sum of t |grad psi . A| / m over the row, over |psi'|."""
     import torch
 
     P, U, B, gamma = _case(name)
@@ -46,7 +47,7 @@ def test_factors_against_oracle(name):
     for k, U0, w in (("l1", tr["UL"], np.ones(P.nnz)), ("l2", tr["U1"], 1.0 - tr["l1"])):
         l, ref = S.export(k), tr[k]
         on = np.ones(P.nnz, bool) if k == "l1" else (S.export("l1") < 1.0) & (tr["l1"] < 1.0)
-        slope = np.full(P.nnz, np.inf)
+        slope, more = np.full(P.nnz, np.inf), np.zeros(P.nnz)
         for r in (rows, P.col_idx):  # |d psi / d l| from either row's side
             q = (1.0 if r is rows else -1.0) * w * ikm[r] * tr["A"]
             V = U0[:, r] + ref * q
@@ -54,5 +55,12 @@ def test_factors_against_oracle(name):
             d = q[-1] - (V[1:-1] * q[1:-1]).sum(0) / V[0] + 0.5 * m2 * q[0] / V[0] ** 2 \
                 - tr["s_min"][r] * gamma * V[0] ** (gamma - 1) * q[0]
             slope = np.minimum(slope, np.abs(d) / V[-1])
-        tol = 1e-14 + 16 * 2.2e-16 / np.maximum(slope, 1e-300)
+            if k == "l2":
+                v = U0[1:-1] / U0[0]
+                grad = np.concatenate([[0.5 * (v * v).sum(0) - tr["s_min"] * gamma * U0[0] ** (gamma - 1)], -v, np.ones((1, P.n))])
+                moved = np.bincount(rows, (tr["l1"] < 1.0) * tol * np.abs((grad[:, rows] * tr["A"]).sum(0)), minlength=P.n) / P.mi
+                more = np.maximum(more, moved[r] / np.maximum(np.abs(d), 1e-300))
+        if k == "l2":
+            more += ref * tol / np.maximum(1.0 - tr["l1"], 1e-300)
+        tol = 1e-14 + 16 * 2.2e-16 / np.maximum(slope, 1e-300) + more
         assert (np.abs(l - ref)[on] <= np.minimum(tol, 1.0)[on]).all(), (k, np.abs(l - ref)[on].max())
