@@ -56,6 +56,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   constexpr int kShared = kMaxBlock + kEll;        // room for one pad slot per element
   using R = std::conditional_t<MX, float, double>;  // arithmetic of steps 1, 2 and the A_ij of step 4
   __shared__ R sR[M][kShared];
+  __shared__ int sE[M][kEll];  // exponent field of the largest right-hand side of each element (FP64 path)
   __shared__ R sdU[M][kShared];
   __shared__ Ctx sctx;
   int lb;
@@ -74,16 +75,19 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   const int sh = t0 + es.l;
   const size_t n = D.n;
   const double tau = stage_tau(c);
+  if constexpr (!MX) {
+    for (int k = threadIdx.x; k < M * kEll; k += blockDim.x) (&sE[0][0])[k] = 0;
+    __syncthreads();
+  }
   const R tau_r = MX ? R(to_f32(tau)) : R(tau);
   double Ui[M];
-  R dUi[M];
+  R rhs[M], dUi[M];
   double Ni = 0.0;
   const bool lim = D.order != GDG_ORDER_HIGH;  // the limiter's steps 3 and 4 follow the solve
   double lo = 0.0, hi = 0.0, sl = 0.0;         // two-hop aggregates of node i (step 3)
   if (valid) {
     load_state<DIM>(U, D.n, i, Ui);
     Ni = abs_bits(S.N[i]);
-    R rhs[M];
 #pragma unroll
     for (int q = 0; q < M; ++q) {
       if constexpr (MX)
@@ -162,7 +166,12 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
       }
     }
 #pragma unroll
-    for (int q = 0; q < M; ++q) sR[q][sh] = rhs[q];
+    for (int q = 0; q < M; ++q) {
+      if constexpr (MX)
+        sR[q][sh] = rhs[q];
+      else
+        atomicMax(&sE[q][es.el], sf::expo(rhs[q]));
+    }
     if (lim) {  // relaxed local bounds, read back after the solve
       double rmin = 0.0, rmax = INFINITY, smin = 0.0;
       if (D.bounds_mode == 0) {
@@ -176,32 +185,58 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
     }
   }
   __syncthreads();
+  if constexpr (!MX) {  // the right-hand sides in fixed point, in the place of the doubles
+    if (valid) {
+#pragma unroll
+      for (int q = 0; q < M; ++q) {
+        const sf::fixp f = sf::fix_parts(sf::fix56(rhs[q], sE[q][es.el]));
+        sR[q][sh] = __hiloint2double(f.hi, f.lo);
+      }
+    }
+    __syncthreads();
+  }
   if (valid) {
     const int nl = D.n_loc;
     const int ei = div_nl(D, i);
     // row il of the element's M_K^{-1}, stored grouped like the entries: (E, a, b) at
     // ((E / kEll * n_loc + a) * n_loc + b) * kEll + E % kEll
-    const double* Minv = D.MKinv + ((size_t)(ei / kEll) * nl + es.l) * nl * kEll + (ei % kEll);
-    R acc[M];
+    const int2* Minv = D.MKinv + ((size_t)(ei / kEll) * nl + es.l) * nl * kEll + (ei % kEll);
+    const int we = D.wexp[i];
+    if constexpr (MX) {
+      R acc[M];
 #pragma unroll
-    for (int q = 0; q < M; ++q) acc[q] = R(0);
-    for (int l = 0; l < nl; ++l) {
-      R w;
-      if constexpr (MX)
-        w = to_f32(Minv[(size_t)l * kEll]);
-      else
-        w = Minv[(size_t)l * kEll];
+      for (int q = 0; q < M; ++q) acc[q] = R(0);
+      for (int l = 0; l < nl; ++l) {
+        const int2 wf = __ldg(Minv + (size_t)l * kEll);
+        const float w = fmaf((float)wf.y, 0x1p-56f, (float)wf.x * 0x1p-28f);  // in units of 2^(we - 1022)
 #pragma unroll
-      for (int q = 0; q < M; ++q) acc[q] += w * sR[q][t0 + l];
+        for (int q = 0; q < M; ++q) acc[q] += w * sR[q][t0 + l];
+      }
+#pragma unroll
+      for (int q = 0; q < M; ++q) dUi[q] = -tau_r * to_f32(sf::mul_pow2(to_f64(acc[q]), we - 1022));
+    } else {
+      // fixed point (fixfp64.cuh): as FP64 multiply-adds this loop held the FP64 pipe, which bounds the kernel, for
+      // 36 of its 162 operations per node (Q2 quads); with the pairs of A below, k_high went from 3.68 to 3.20 ms
+      // per launch at Q2 1024^2 and from 555 to 488 us at Q1 48 x 40 x 44
+      sf::fixs s[M];
+#pragma unroll
+      for (int q = 0; q < M; ++q) s[q] = sf::fixs{0, 0, 0};
+      for (int l = 0; l < nl; ++l) {
+        const int2 wf = __ldg(Minv + (size_t)l * kEll);
+#pragma unroll
+        for (int q = 0; q < M; ++q) {
+          const double r = sR[q][t0 + l];
+          sf::fix_mad(sf::fixp{wf.x, wf.y}, sf::fixp{__double2hiint(r), __double2loint(r)}, s[q]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < M; ++q) {
+        const int re = sE[q][es.el];
+        dUi[q] = re < 0x7ff ? sf::mul(sf::neg(tau), sf::fix_dbl(s[q], we, re)) : __longlong_as_double(0x7ff8000000000000LL);
+      }
     }
 #pragma unroll
-    for (int q = 0; q < M; ++q) {
-      if constexpr (MX)
-        dUi[q] = -tau_r * acc[q];
-      else
-        dUi[q] = -tau * acc[q];
-      sdU[q][sh] = dUi[q];
-    }
+    for (int q = 0; q < M; ++q) sdU[q][sh] = dUi[q];
     if (D.order == GDG_ORDER_HIGH) {
 #pragma unroll
       for (int q = 0; q < M; ++q) {
@@ -216,10 +251,51 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   }
   if (D.order == GDG_ORDER_HIGH) return;
   __syncthreads();
+  const int nl = D.n_loc;
+  const int se = valid ? D.sten_end[i] : 0, r0 = valid ? D.rbeg[i] : 0, r1 = valid ? D.rend[i] : 0;
+  // Antidiffusive fluxes.  The mass term couples the nodes of one element, and A_ji = -A_ij: each pair is worked
+  // out once, by the node that has at most half the element after it (cyclically), and stored at both
+  // entries; half the FP64 operations of a loop in which every row does its own.
+  const int elem = valid ? div_nl(D, i) : 0;
+  for (int e = r0; e < r1; e += kEll) {
+    const int j = D.col[e];
+    const bool stencil = e < se;
+    const int ej = div_nl(D, j);
+    if (ej != elem) {  // no mass term
+      if (!stencil)
+#pragma unroll
+        for (int q = 0; q < M; ++q) S.A[(size_t)q * D.nnz + e] = 0.0;
+      continue;
+    }
+    const int lj = j - ej * nl;
+    int after = lj - es.l;
+    if (after < 0) after += nl;
+    if (2 * after > nl || (2 * after == nl && lj < es.l)) continue;
+    const int t = D.tr[e];
+    if constexpr (MX) {
+      const float mij = to_f32(D.mij[e]);
+#pragma unroll
+      for (int q = 0; q < M; ++q) {
+        const float a = stencil ? to_f32(S.A[(size_t)q * D.nnz + e]) : 0.f;
+        const double v = to_f64(fmaf(-mij, sdU[q][t0 + lj] - dUi[q], a));
+        S.A[(size_t)q * D.nnz + e] = v;
+        S.A[(size_t)q * D.nnz + t] = sf::neg(v);
+      }
+    } else {
+      const double mij = D.mij[e];
+#pragma unroll
+      for (int q = 0; q < M; ++q) {
+        const double a = stencil ? S.A[(size_t)q * D.nnz + e] : 0.0;
+        const double v = fma(-mij, sdU[q][t0 + lj] - dUi[q], a);
+        S.A[(size_t)q * D.nnz + e] = v;
+        S.A[(size_t)q * D.nnz + t] = sf::neg(v);
+      }
+    }
+  }
+  __syncthreads();
   if (!valid) return;
   const double rmin = S.bounds[i], rmax = S.bounds[n + i], smin = S.bounds[2 * n + i];
-  const int se = D.sten_end[i];
-  // antidiffusive fluxes and pass-1 line search
+  // pass-1 line search
   double UL[M];
 #pragma unroll
   for (int q = 0; q < M; ++q) UL[q] = S.UL[(size_t)q * n + i];
@@ -227,34 +303,10 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   ls_row<DIM>(D, ls, UL, rmin, rmax, smin);
   const double ikm = D.inv_km[i];
   const float ikmf = d2f_fast(ikm);
-  const int nl = D.n_loc;
-  const int elem = div_nl(D, i);
-  for (int e = D.rbeg[i], e1 = D.rend[i]; e < e1; e += kEll) {
-    int j = D.col[e];
+  for (int e = r0; e < r1; e += kEll) {
     double A[M];
-    const bool stencil = e < se;
-    const int ej = div_nl(D, j);
-    const bool same = ej == elem;
-    const int tj = t0 + (j - ej * nl);
-    if constexpr (MX) {
-      const float mij = same ? to_f32(D.mij[e]) : 0.f;
 #pragma unroll
-      for (int q = 0; q < M; ++q) {
-        float a = stencil ? to_f32(S.A[(size_t)q * D.nnz + e]) : 0.f;
-        if (same) a = fmaf(-mij, sdU[q][tj] - dUi[q], a);
-        A[q] = to_f64(a);
-        S.A[(size_t)q * D.nnz + e] = A[q];
-      }
-    } else {
-      const double mij = same ? D.mij[e] : 0.0;
-#pragma unroll
-      for (int q = 0; q < M; ++q) {
-        double a = stencil ? S.A[(size_t)q * D.nnz + e] : 0.0;
-        if (same) a = fma(-mij, sdU[q][tj] - dUi[q], a);
-        A[q] = a;
-        S.A[(size_t)q * D.nnz + e] = a;
-      }
-    }
+    for (int q = 0; q < M; ++q) A[q] = S.A[(size_t)q * D.nnz + e];
     // A = 0 (a uniform neighbourhood): the search's outcome is l = 1 exactly when the FP32 tests it
     // starts with pass, which here reduce to a density gap above and psi(0) > 0; then skip them
     unsigned long long abits = 0;

@@ -176,6 +176,8 @@ SF_FN double mul(double a, double b) {
   return dbl2(rh, rl);
 }
 
+SF_FN double neg(double x) { return dbl2(hiw(x) ^ 0x80000000u, low(x)); }
+
 // x * 2^k for -1022 <= k <= 1023 by adding k to the exponent field: exact for a normal x whose scaled
 // value is normal, and for zeros; every other case takes the FP64 instruction.
 SF_FN double mul_pow2(double x, int k) {
@@ -231,6 +233,6 @@ SF_FN double add(double a, double b) {
   return dbl2(rh, rl);
 }
 
-SF_FN double sub(double a, double b) { return add(a, dbl2(hiw(b) ^ 0x80000000u, low(b))); }
+SF_FN double sub(double a, double b) { return add(a, neg(b)); }
 
 }  // namespace sf
