@@ -61,6 +61,20 @@ def bytes_per_launch(c: Counts) -> dict:
     )
 
 
+def quiet_bytes_per_launch(c: Counts) -> dict:
+    """bytes_per_launch of a mesh on which every state is the same: the edge sweep stores d_ij alone, sweep A reads nothing else
+    of an entry but its column, the element sweep writes bounds and factors but no A, and sweep C reads no entry."""
+    m, d, n, nnz, s = c.m, c.dim, c.n, c.nnz, c.nnz_s
+    rowptr = 4 * (n + 1)
+    out = bytes_per_launch(c)
+    out["edge"] = (s // 2) * (4 * 4 + 8 * (1 + d)) + 8 * (m + 5) * n + s * 8
+    out["low"] = 8 * m * n + 8 * 4 * n + rowptr + s * (4 + 8) + 8 * (2 * m + 1 + 3) * n
+    out["high"] = 8 * m * n * 2 + rowptr + s * 4 + 8 * 3 * n * 2 + 8 * n + 8 * nnz + n
+    out["limit2"] = rowptr + 8 * m * n * 2 + 2 * n
+    out["final"] = 8 * m * n * 3 + n
+    return out
+
+
 def flops_per_launch(c: Counts) -> dict:
     m, d, n, nnz, s, nb, nl = c.m, c.dim, c.n, c.nnz, c.nnz_s, c.nb, c.n_loc
     lam = 28  # wave-speed bound from the per-node primitives

@@ -1036,6 +1036,15 @@ int gdg_debug_export(gdg_handle* h, const char* name, double* dst, int64_t count
   if (kind == 0 && per_entry) {  // device entry order back to the caller's
     for (int64_t r = 0; r < want / std::max<int64_t>(nnz, 1); ++r)
       for (int64_t q = 0; q < nnz; ++q) dst[r * nnz + h->eorig[q]] = tmp[r * NE + h->epos[q]];
+    if (nm == "A" && h->D.order == GDG_ORDER_LIMITED && h->D.passes > 0) {  // rows whose A is zero are not stored
+      std::vector<unsigned char> rem(n);
+      if (n > 0 && (e = cudaMemcpy(rem.data(), h->S.rem, n, cudaMemcpyDeviceToHost)) != cudaSuccess)
+        return cuda_fail(e);
+      for (int64_t i = 0; i < n; ++i)
+        if (rem[i] == 2)
+          for (int64_t q = h->row_ptr[i]; q < h->row_ptr[i + 1]; ++q)
+            for (int64_t r = 0; r < m; ++r) dst[r * nnz + h->eorig[q]] = 0.0;
+    }
   } else if (kind == 0) {
     std::memcpy(dst, tmp.data(), sizeof(double) * want);
   } else if (kind == 1) {

@@ -167,7 +167,8 @@ struct Scratch {
   double* l2;      // [nnz] pass 2
   double* l2B;     // [nb]
   double* U1;      // [m][n]
-  unsigned char* rem;  // [n] 1 where row i has a pass-2 remainder (a symmetrised pass-1 factor below 1)
+  unsigned char* rem;  // [n] from the element sweep: 2 where all of row i's A is zero and therefore not stored; then from
+                       // sweep C also 1 where the row has a pass-2 remainder (a symmetrised pass-1 factor below 1)
   unsigned int* flags;
   unsigned int* lsq_n;  // [2] lengths of the deferred line-search queues of passes 1 and 2
   int2* lsq;            // [nnz + nb] deferred line searches of the current pass (ls_defer)
@@ -497,6 +498,13 @@ __device__ __forceinline__ double f2d_fast(float f) {
 __device__ __forceinline__ double abs_bits(double x) {
   return __longlong_as_double(__double_as_longlong(x) & 0x7fffffffffffffffLL);
 }
+__device__ __forceinline__ bool same_bits(double x, double y) {
+  return __double_as_longlong(x) == __double_as_longlong(y);
+}
+// x or'ed into a mask that stays zero while every x is +-0
+__device__ __forceinline__ void nonzero_bits(unsigned& mask, double x) {
+  mask |= ((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x);
+}
 __device__ __forceinline__ bool is_zero_bits(double x) { return (__double_as_longlong(x) << 1) == 0; }
 __device__ __forceinline__ bool is_one_bits(double x) { return __double_as_longlong(x) == 0x3ff0000000000000LL; }
 
@@ -567,6 +575,8 @@ __device__ __forceinline__ double lambda_max(const Dev& D, double uL, double pL,
   // max(x, 0), the tests x > 0 and the final maximum of two non-negative values on the integer pipe
   // (a positive double is a positive int64)
   auto pos = [](double x) { return __double_as_longlong(x) > 0 ? x : 0.0; };
+  // equal states (all of a region that no wave has reached): p~ = p, and the waves move at u -+ a
+  if (same_bits(uL, uR) & same_bits(pL, pR) & same_bits(aL, aR)) return pmax(pos(aL - uL), pos(uR + aR));
   double num = pos(fma(-D.gm1h, uR - uL, aL + aR));
   const double den = fma(aL, pmeL, sf::mul(aR, pmeR));
   double pt;  // (num / den)^{1/e}

@@ -56,7 +56,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   constexpr int kShared = kMaxBlock + kEll;        // room for one pad slot per element
   using R = std::conditional_t<MX, float, double>;  // arithmetic of steps 1, 2 and the A_ij of step 4
   __shared__ R sR[M][kShared];
-  __shared__ int sE[M][kEll];  // exponent field of the largest right-hand side of each element (FP64 path)
+  __shared__ int sE[M][kEll];  // exponent field of the largest right-hand side of each element, 0 where all are zero
   __shared__ R sdU[M][kShared];
   __shared__ Ctx sctx;
   int lb;
@@ -75,16 +75,16 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   const int sh = t0 + es.l;
   const size_t n = D.n;
   const double tau = stage_tau(c);
-  if constexpr (!MX) {
-    for (int k = threadIdx.x; k < M * kEll; k += blockDim.x) (&sE[0][0])[k] = 0;
-    __syncthreads();
-  }
+  for (int k = threadIdx.x; k < M * kEll; k += blockDim.x) (&sE[0][0])[k] = 0;
+  __syncthreads();
   const R tau_r = MX ? R(to_f32(tau)) : R(tau);
   double Ui[M];
   R rhs[M], dUi[M];
   double Ni = 0.0;
   const bool lim = D.order != GDG_ORDER_HIGH;  // the limiter's steps 3 and 4 follow the solve
   double lo = 0.0, hi = 0.0, sl = 0.0;         // two-hop aggregates of node i (step 3)
+  bool quiet = true;                           // no viscous part of A in the row, and no boundary entry
+  unsigned zeros = 0;                          // the stencil entries (of the row's first 32) without a viscous part
   if (valid) {
     load_state<DIM>(U, D.n, i, Ui);
     Ni = abs_bits(S.N[i]);
@@ -106,10 +106,10 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
     }
     // not unrolled: with its products on the integer pipe the loop body is large, and unrolled by 2 the
     // kernel stalled on instruction fetch (4.24 against 4.14 ms per launch at Q2 1024^2)
+    unsigned bit = 1;  // of the entry in zeros; 0 from the row's 33rd entry on
 #pragma unroll 1
-    for (int e = D.rbeg[i]; e < e1; e += kEll) {  // I(i)
+    for (int e = D.rbeg[i]; e < e1; e += kEll, bit <<= 1) {  // I(i)
       const int j = __ldg(D.col + e);
-      const double dl64 = __ldg(S.dL + e), mu = __ldg(D.mu + e), Nj = abs_bits(__ldg(S.N + j));
       double Uj[M];
 #pragma unroll
       for (int q = 0; q < M; ++q) Uj[q] = __ldg(U + (size_t)q * n + j);
@@ -118,6 +118,18 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
         hi = pmax(hi, __ldg(S.agg + n + j));
         sl = pmin(sl, __ldg(S.agg + 2 * n + j));
       }
+      bool same = true;
+#pragma unroll
+      for (int q = 0; q < M; ++q) same = same && same_bits(Ui[q], Uj[q]);
+      if (same) {  // no viscous term; its zero is stored only where a row with other terms needs it
+        zeros |= bit;
+        if (bit == 0)
+#pragma unroll
+          for (int q = 0; q < M; ++q) S.A[(size_t)q * D.nnz + e] = 0.0;
+        continue;
+      }
+      quiet = false;
+      const double dl64 = __ldg(S.dL + e), mu = __ldg(D.mu + e), Nj = abs_bits(__ldg(S.N + j));
       if constexpr (MX) {
         // d^H - d^L from FP32 operands: every factor is symmetric in (i, j), so the same bits come out
         // of row j, and A_ji = -A_ij holds exactly
@@ -146,6 +158,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
       }
     }
     for (int b = D.b_ptr[i]; b < D.b_ptr[i + 1]; ++b) {
+      quiet = false;
       if (lim) {
         lo = pmin(lo, S.bbar[b]);
         hi = pmax(hi, S.bbar[b]);
@@ -167,10 +180,14 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
     }
 #pragma unroll
     for (int q = 0; q < M; ++q) {
-      if constexpr (MX)
+      int ex;
+      if constexpr (MX) {
         sR[q][sh] = rhs[q];
-      else
-        atomicMax(&sE[q][es.el], sf::expo(rhs[q]));
+        ex = (int)(__float_as_uint(rhs[q]) & 0x7fffffffu);
+      } else {
+        ex = sf::expo(rhs[q]);
+      }
+      if (ex > 0) atomicMax(&sE[q][es.el], ex);
     }
     if (lim) {  // relaxed local bounds, read back after the solve
       double rmin = 0.0, rmax = INFINITY, smin = 0.0;
@@ -185,8 +202,12 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
     }
   }
   __syncthreads();
+  // all right-hand sides of the element zero: so are dU^H and the mass terms of A
+  bool flat = true;
+#pragma unroll
+  for (int q = 0; q < M; ++q) flat = flat && sE[q][es.el] == 0;
   if constexpr (!MX) {  // the right-hand sides in fixed point, in the place of the doubles
-    if (valid) {
+    if (valid && !flat) {
 #pragma unroll
       for (int q = 0; q < M; ++q) {
         const sf::fixp f = sf::fix_parts(sf::fix56(rhs[q], sE[q][es.el]));
@@ -202,13 +223,17 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
     // ((E / kEll * n_loc + a) * n_loc + b) * kEll + E % kEll
     const int2* Minv = D.MKinv + ((size_t)(ei / kEll) * nl + es.l) * nl * kEll + (ei % kEll);
     const int we = D.wexp[i];
-    if constexpr (MX) {
+    if (flat) {
+#pragma unroll
+      for (int q = 0; q < M; ++q) dUi[q] = R(0);
+    } else if constexpr (MX) {
       R acc[M];
 #pragma unroll
       for (int q = 0; q < M; ++q) acc[q] = R(0);
       for (int l = 0; l < nl; ++l) {
         const int2 wf = __ldg(Minv + (size_t)l * kEll);
-        const float w = fmaf((float)wf.y, 0x1p-56f, (float)wf.x * 0x1p-28f);  // in units of 2^(we - 1022)
+        // in units of 2^(we - 1022), truncated like to_f32
+        const float w = __ll2float_rz(((long long)wf.x << 28) + wf.y) * 0x1p-56f;
 #pragma unroll
         for (int q = 0; q < M; ++q) acc[q] += w * sR[q][t0 + l];
       }
@@ -256,13 +281,24 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   // Antidiffusive fluxes.  The mass term couples the nodes of one element, and A_ji = -A_ij: each pair is worked
   // out once, by the node that has at most half the element after it (cyclically), and stored at both
   // entries; half the FP64 operations of a loop in which every row does its own.
+  // With dU^H = 0 the viscous part, which both rows have, is all there is; a row whose A is zero throughout is
+  // marked instead of written: U^(1)_i = U^L_i whatever its factors, which are 1.
   const int elem = valid ? div_nl(D, i) : 0;
-  for (int e = r0; e < r1; e += kEll) {
+  quiet = quiet && flat;
+  if (flat && !quiet) {
+    unsigned bit = 1;
+    for (int e = r0; e < r1; e += kEll, bit <<= 1)
+      if (e >= se || (zeros & bit))
+#pragma unroll
+        for (int q = 0; q < M; ++q) S.A[(size_t)q * D.nnz + e] = 0.0;
+  }
+  unsigned bit = 1;
+  for (int e = flat ? r1 : r0; e < r1; e += kEll, bit <<= 1) {
     const int j = D.col[e];
-    const bool stencil = e < se;
+    const bool visc = e < se && !(zeros & bit);
     const int ej = div_nl(D, j);
     if (ej != elem) {  // no mass term
-      if (!stencil)
+      if (!visc)
 #pragma unroll
         for (int q = 0; q < M; ++q) S.A[(size_t)q * D.nnz + e] = 0.0;
       continue;
@@ -276,7 +312,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
       const float mij = to_f32(D.mij[e]);
 #pragma unroll
       for (int q = 0; q < M; ++q) {
-        const float a = stencil ? to_f32(S.A[(size_t)q * D.nnz + e]) : 0.f;
+        const float a = visc ? to_f32(S.A[(size_t)q * D.nnz + e]) : 0.f;
         const double v = to_f64(fmaf(-mij, sdU[q][t0 + lj] - dUi[q], a));
         S.A[(size_t)q * D.nnz + e] = v;
         S.A[(size_t)q * D.nnz + t] = sf::neg(v);
@@ -285,7 +321,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
       const double mij = D.mij[e];
 #pragma unroll
       for (int q = 0; q < M; ++q) {
-        const double a = stencil ? S.A[(size_t)q * D.nnz + e] : 0.0;
+        const double a = visc ? S.A[(size_t)q * D.nnz + e] : 0.0;
         const double v = fma(-mij, sdU[q][t0 + lj] - dUi[q], a);
         S.A[(size_t)q * D.nnz + e] = v;
         S.A[(size_t)q * D.nnz + t] = sf::neg(v);
@@ -294,6 +330,11 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   }
   __syncthreads();
   if (!valid) return;
+  S.rem[i] = quiet ? 2 : 0;
+  if (quiet) {
+    for (int e = r0; e < r1; e += kEll) S.l1[e] = 1.0;
+    return;
+  }
   const double rmin = S.bounds[i], rmax = S.bounds[n + i], smin = S.bounds[2 * n + i];
   // pass-1 line search
   double UL[M];

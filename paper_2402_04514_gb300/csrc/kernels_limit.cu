@@ -29,7 +29,8 @@ __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last
   double acc[M];
 #pragma unroll
   for (int q = 0; q < M; ++q) acc[q] = 0.0;
-  const int r0 = D.rbeg[i], r1 = D.rend[i];
+  const bool quiet = S.rem[i] == 2;  // all of A is zero (and not stored): no sum
+  const int r0 = D.rbeg[i], r1 = quiet ? r0 : D.rend[i];
   bool remainder = false;  // some entry has l1 < 1, so that pass 2 has a remainder to limit
   for (int e = r0; e < r1; e += kEll) {
     double l = pmin(S.l1[e], S.l1[D.tr[e]]);  // limiter coefficients are in [0, 1]: integer min
@@ -54,7 +55,7 @@ __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last
   }
 #pragma unroll
   for (int q = 0; q < M; ++q) S.U1[q * n + i] = U1[q];
-  S.rem[i] = remainder;
+  S.rem[i] = quiet ? 2 : remainder;
   // l2 is computed only where it multiplies a nonzero remainder (1 - l1)A: k_final reads no other, and a
   // row without a remainder (the flag above) takes no row context and no search
   if (!remainder) return;
@@ -152,7 +153,7 @@ __device__ __forceinline__ void final_body(const Src& src, int sliced) {
   const int i = row_node(D, lb * blockDim.x + threadIdx.x, sliced && !c.Uhost);
   if (i < 0) return;
   const size_t n = D.n, nnz = D.nnz, nb = D.nb;
-  if (!S.rem[i]) {  // no remainder in the row: U^(2)_i = U^(1)_i
+  if (S.rem[i] != 1) {  // no remainder in the row: U^(2)_i = U^(1)_i
 #pragma unroll
     for (int q = 0; q < M; ++q) store_out(c, q * n + i, rk_out(c, q * n + i, S.U1[q * n + i]));
     return;

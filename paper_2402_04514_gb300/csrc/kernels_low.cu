@@ -213,6 +213,18 @@ __global__ void __maxnreg__(48) k_tau(Src src, int sliced) {
   tau_body<DIM, MX, Src>(src, sliced);
 }
 
+// s~ of a state in the mixed path, from rho, |m|^2 / 2 and E: eps in FP64 (E - |m|^2 / (2 rho) cancels at high Mach
+// numbers) with 1/rho from one Newton step on the FP32 reciprocal; rho^{-gamma} in FP32.
+__device__ __forceinline__ double entropy_mx(const Dev& D, double rho, double hm2, double E) {
+  const float rf = to_f32(rho);
+  const double y = to_f64(1.f / rf);
+  double ir = __dmul_rn(y, fma(-rho, y, 2.0));
+  const float rg = powf(rf, -D.gamma_f);
+  if (finite_f32(rg)) return to_f64(__fmul_rn(rg, to_f32(fma(-hm2, ir, E))));
+  const double rg64 = rho_neg_gamma(D, rho, &ir);
+  return rg64 * fma(-hm2, ir, E);
+}
+
 // What a stage needs of boundary entry b, one thread per entry (the first threads of the edge sweep, so that
 // the sweeps over rows read it instead of working it out inside their rows: the powers, roots and
 // divisions of an entry are a chain of FP64 operations that held up its row's whole warp, in every sweep
@@ -318,6 +330,15 @@ __device__ __forceinline__ void edge_body(const Src& src) {
   const double d = sf::mul(cnm, lam);
   S.dL[e] = d;
   S.dL[t] = d;
+  // Equal states, as in every region that no wave has reached: the differences are zero and the bar state is the
+  // state itself, so the sweeps over rows, which see it from the states, take nothing but d_ij from the entry.
+  // In ms per launch at Q2 1024^2, where the waves have crossed a few percent of the mesh: k_edge 2.22 -> 0.95, k_low
+  // 1.89 -> 0.97, k_high 3.20 -> 1.51, k_limit2 0.96 -> 0.51.  Where no two states agree the tests cost 2% of a
+  // step (Q1 512^2 vortex: k_high 237 -> 246 us, k_edge 196 -> 199, k_low 187 -> 183).
+  bool same = true;
+#pragma unroll
+  for (int q = 0; q < M; ++q) same = same && same_bits(Ui[q], Uj[q]);
+  if (same) return;
   // f(U) c_ij with c_ij = |c_ij| n_ij, from m.c = |c| m.n and v.c = |c| v.n
   double cv[DIM], gi[M], gj[M];
 #pragma unroll
@@ -345,24 +366,15 @@ __device__ __forceinline__ void edge_body(const Src& src) {
   double Ub[M];
   Ub[0] = sf::mul_pow2(W[0], -1);
   Ub[DIM + 1] = sf::mul_pow2(W[DIM + 1], -1);
-  double mw2 = sf::mul(W[1], W[1]), irb;  // |2 m(Ubar)|^2; 0.125 mw2 = |m(Ubar)|^2 / 2
+  double mw2 = sf::mul(W[1], W[1]);  // |2 m(Ubar)|^2; 0.125 mw2 = |m(Ubar)|^2 / 2
 #pragma unroll
   for (int q = 1; q < DIM; ++q) mw2 = fma(W[1 + q], W[1 + q], mw2);
   const double hm2 = sf::mul_pow2(mw2, -3);
   double stb;
   if constexpr (MX) {
-    // eps(Ubar) in FP64 (E - |m|^2 / (2 rho) cancels at high Mach numbers) with 1/rho(Ubar) from one
-    // Newton step on the FP32 reciprocal; rho(Ubar)^{-gamma} in FP32
-    const float rbf = to_f32(Ub[0]);
-    const double y = to_f64(1.f / rbf);
-    irb = y * fma(-Ub[0], y, 2.0);
-    const float rg = powf(rbf, -D.gamma_f);
-    stb = to_f64(rg * to_f32(fma(-hm2, irb, Ub[DIM + 1])));
-    if (!finite_f32(rg)) {
-      const double rgb = rho_neg_gamma(D, Ub[0], &irb);
-      stb = rgb * fma(-hm2, irb, Ub[DIM + 1]);
-    }
+    stb = entropy_mx(D, Ub[0], hm2, Ub[DIM + 1]);
   } else {
+    double irb;
     const double rgb = rho_neg_gamma(D, Ub[0], &irb);  // sets irb = 1 / rho(Ubar) before its use below
     stb = sf::mul(rgb, fma(-hm2, irb, Ub[DIM + 1]));
   }
@@ -425,12 +437,22 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
   double lo = Ui[0], hi = Ui[0], sl = st_i;
   const size_t nnz = D.nnz;
   const int e1 = D.sten_end[i];
+  bool active = D.b_ptr[i + 1] > D.b_ptr[i];  // some sum of the row has a term that is not zero
+  bool equal = false;                         // some neighbour has the row's state
   for (int e = D.rbeg[i]; e < e1; e += kEll) {  // I(i)
     const int j = D.col[e];
     const double d = S.dL[e];
     dsum += d;
     double Uj[M];
     load_state<DIM>(U, D.n, j, Uj);
+    bool same = true;
+#pragma unroll
+    for (int q = 0; q < M; ++q) same = same && same_bits(Ui[q], Uj[q]);
+    if (same) {  // equal states: the edge sweep's terms are zeros, and the extrema stay
+      equal = true;
+      continue;
+    }
+    active = true;
 #pragma unroll
     for (int q = 0; q < M; ++q) {
       const double ge = S.G[q * nnz + e];
@@ -445,6 +467,10 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
     lo = pmin(lo, pmin(Uj[0], S.barR[e]));
     hi = pmax(hi, pmax(Uj[0], S.barR[e]));
     sl = pmin(sl, S.barS[e]);
+  }
+  if constexpr (MX) {
+    // the bar state of equal states is the state, but its s~ is rounded otherwise in FP32 than k_prim's
+    if (equal) sl = pmin(sl, entropy_mx(D, Ui[0], sf::mul_pow2(dot<DIM>(Ui + 1, Ui + 1), -1), Ui[DIM + 1]));
   }
   // sg is now the sum of (f(U_j) - f(U_i)) c_ij; with the boundary terms, Fsum = sg - f(U_i) sum_k c_i^{d,k} =
   // sum_j f(U_j) c_ij and the right-hand side takes Fsum + sum_k f(U^{d,k}) c_i^{d,k}.  On a stencil that
@@ -467,12 +493,17 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
   }
   const double inv_mi = D.inv_mi[i];
   if (sf::mul(sf::mul(sf::mul_pow2(tau, 1), dsum), inv_mi) > 1.0 + 1e-12) atomicOr(S.flags, (unsigned)GDG_FLAG_CFL);
-  double rhs[M];
+  double rhs[M], UL[M];
 #pragma unroll
-  for (int q = 0; q < M; ++q) rhs[q] = (sg[q] + sgB[q]) - sdu[q];
-  double UL[M];
+  for (int q = 0; q < M; ++q) rhs[q] = 0.0, UL[q] = Ui[q];
+  if (active) {
+    const double tm = -sf::mul(tau, inv_mi);
 #pragma unroll
-  for (int q = 0; q < M; ++q) UL[q] = fma(-sf::mul(tau, inv_mi), rhs[q], Ui[q]);
+    for (int q = 0; q < M; ++q) {
+      rhs[q] = (sg[q] + sgB[q]) - sdu[q];
+      UL[q] = fma(tm, rhs[q], Ui[q]);
+    }
+  }
   if (write_out) {
 #pragma unroll
     for (int q = 0; q < M; ++q) store_out(c, (size_t)q * n + i, rk_out(c, (size_t)q * n + i, UL[q]));
@@ -486,6 +517,10 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
   S.agg[i] = lo;
   S.agg[n + i] = hi;
   S.agg[2 * n + i] = sl;
+  if (!active) {
+    S.N[i] = 0.0;
+    return;
+  }
   // entropy-viscosity indicator: Fsum_k = sum_j (f_k(U_j) - f_k(U_i)) c_ij - f_k(U_i) sum_k c_i^{d,k}, which
   // equals sum_j f_k(U_j) c_ij by the partition of unity (Lemma LemPart) and vanishes exactly on a
   // stencil holding one state; grad Phi_i = rho_i f'(s_i) grad_U s(U_i), f' = f / (gamma + 1),
