@@ -844,13 +844,12 @@ __device__ __forceinline__ void boundary_state(const Dev& D, int b, const double
 }
 
 // Per-row context of the line searches from one state U0 (the row's U^L or U^(1)) against the row's
-// bounds: psi(0) in FP64 once per row, and FP32 copies of U0's parts, of psi(0) and of the distances of
-// rho(U0) to its bounds for the FP32 certificates.  The searches run along P = w A (w = the row's
-// 1 / (kappa_i m_i), times 1 - l1 in pass 2), so a point t of the search is U0 + (t w) A.
+// bounds: FP32 copies of U0's parts, of psi(0), worked out in FP64, and of the distances of rho(U0) to its
+// bounds, for the FP32 certificates.  The searches run along P = w A (w = the row's 1 / (kappa_i m_i), times
+// 1 - l1 in pass 2), so a point t of the search is U0 + (t w) A.
 template <int DIM>
 struct LsRow {
-  double U0[DIM + 2];
-  double rmin, rmax, smin, psi0;
+  double rho, rmin, rmax;
   float r0, ir0, m0[DIM], m0sq, sg0, psi0f, dlo, dhi;
   float fl;  // min(rho0, |m0_k|, psi0f) in FP32, 0 unless all are positive: the bound of d2f_incr's guard
 };
@@ -858,22 +857,20 @@ struct LsRow {
 template <int DIM>
 __device__ __forceinline__ void ls_row(const Dev& D, LsRow<DIM>& c, const double* U0, double rmin, double rmax,
                                        double smin) {
-#pragma unroll
-  for (int q = 0; q < DIM + 2; ++q) c.U0[q] = U0[q];
   const double m2 = dot_fp64<DIM>(U0 + 1, U0 + 1);
+  c.rho = U0[0];
   c.rmin = rmin;
   c.rmax = rmax;
-  c.smin = smin;
   double ir;
   double rg = (U0[0] > 0.0) ? rho_pow_gamma(D, U0[0], &ir) : 0.0;
-  c.psi0 = (U0[0] > 0.0) ? fma(-smin, rg, fma(-sf::mul_pow2(m2, -1), ir, U0[DIM + 1])) : -1.0;
+  const double psi0 = (U0[0] > 0.0) ? fma(-smin, rg, fma(-sf::mul_pow2(m2, -1), ir, U0[DIM + 1])) : -1.0;
   c.r0 = d2f_fast(U0[0]);
   c.ir0 = __frcp_rn(c.r0);
 #pragma unroll
   for (int k = 0; k < DIM; ++k) c.m0[k] = d2f_fast(U0[1 + k]);
   c.m0sq = d2f_fast(m2);
   c.sg0 = d2f_fast(smin * rg);
-  c.psi0f = d2f_fast(c.psi0);
+  c.psi0f = d2f_fast(psi0);
   // distances to the density bounds for the FP32 density certificate, kept only when they exceed 1e-6
   // rho(U0): the FP64 comparisons of the closed form round relative to rho, so a certificate on a smaller
   // gap could disagree with them (a zero distance sends every search of the row to the FP64 form)
@@ -962,43 +959,43 @@ __device__ __forceinline__ bool ls_certified(const Dev& D, const LsRow<DIM>& c, 
   return t > 1e-4f * scale + 1e-6f * fabsf(c.psi0f);
 }
 
-// Largest l in [0, 1] with U0 + l P in B_i, P = w A (Sec. 5.4, eq. (ConvexScheme), Lemma
-// ConsInvariants), in two parts.  The head takes the closed form for the density bounds and decides the
-// common cases: the entropy constraint holds at l_rho (proved by the FP32 certificate, else by psi in FP64),
-// or psi(0) < 0 (roundoff) and l = 0.  It returns false when psi(l_rho) < 0 <= psi(0): then the tail looks for
-// the root in between and returns a feasible point within ls_tol, or psi's rounding, of it.  The FP32
-// certificate only skips FP64 evaluations whose outcome it proves.
+// The largest factor that the density bounds allow, in closed form, Pr = w A_rho.
+__device__ __forceinline__ double ls_density(double rho, double Pr, double rmin, double rmax) {
+  const double r1 = rho + Pr;
+  double l = 1.0;
+  if (r1 < rmin) l = sf::mul(rmin - rho, rcp64(Pr));
+  if (r1 > rmax) l = sf::mul(rmax - rho, rcp64(Pr));
+  if (__double_as_longlong(l) <= 0) l = 0.0;  // comparisons with 0 and 1 on the integer pipe
+  return pmin(l, 1.0);
+}
+
+// Largest l in [0, 1] with U0 + l P in B_i, P = w A (Sec. 5.4, eq. (ConvexScheme), Lemma ConsInvariants), as far as it
+// takes no FP64 evaluation of psi: l_rho = 1 where FP32 proves rho(U0) + P_rho inside [rho_min, rho_max], else from
+// the closed form, and true where the FP32 certificate proves psi(l_rho) >= 0.  Every other search is queued
+// (ls_defer) and solved by line_search: a few entries of a row in the wavefronts, but hardly a warp there is
+// without one, and evaluated here each held up its warp, with one or two lanes at work, on the pipe that
+// bounds the kernel.  In us per launch at Q1 48 x 40 x 44: k_high 505 -> 396, k_limit2 284 -> 175, k_lsfix 249 -> 171 (its
+// own products and comparisons moved to FP32 and the integer pipe as well).  With the density-limited searches queued
+// too, k_high took 385 and k_limit2 161, but k_lsfix 430: a queued item is some 16 scattered loads.
+//
+// The density test (wf = w in FP32): the products and conversions have relative error below 4e-7, so a
+// relative margin of 1e-6 on both sides leaves the exact distance to the bound above 8e-7 times a gap
+// of at least 1e-6 rho (ls_row), far beyond the FP64 rounding of the closed form's comparisons, which
+// therefore agree with it.  An A_rho below the FP32 range counts as 0 under the guard of d2f_incr, which
+// also makes rho(U0) + w A_rho round to rho(U0) in the closed form.
 template <int DIM>
-__device__ __forceinline__ bool line_search_head(const Dev& D, const LsRow<DIM>& c, const double* A, double w,
-                                                 float wf, double* l_out, double* fb_out) {
-  // Density bounds.  The common case, rho(U0) + w A_rho inside [rho_min, rho_max] so that l_rho = 1, is
-  // proved in FP32 (wf = w in FP32): the products and conversions have relative error below 4e-7, so a
-  // relative margin of 1e-6 on both sides leaves the exact distance to the bound above 8e-7 times a gap
-  // of at least 1e-6 rho (ls_row), far beyond the FP64 rounding of the closed form's comparisons, which
-  // therefore agree with it.  An A_rho below the FP32 range counts as 0 under the guard of d2f_incr, which
-  // also makes rho(U0) + w A_rho round to rho(U0) in the closed form.
+__device__ __forceinline__ bool line_search_sure(const Dev& D, const LsRow<DIM>& c, const double* A, double w, float wf,
+                                                 double* l_out) {
   const float pr = wf * d2f_incr(A[0], wf * 0x1p-71f < c.fl);
   const bool inside = pr >= 0.f ? pr * 1.000001f < c.dhi * 0.999999f : -pr * 1.000001f < c.dlo * 0.999999f;
   double l = 1.0;
-  float sf = wf;
+  float at = wf;
   if (!inside) {
-    const double Pr = __dmul_rn(w, A[0]);
-    if (c.U0[0] + Pr < c.rmin) l = (c.rmin - c.U0[0]) / Pr;
-    if (c.U0[0] + Pr > c.rmax) l = (c.rmax - c.U0[0]) / Pr;
-    if (!(l > 0.0)) l = 0.0;
-    if (l > 1.0) l = 1.0;
-    sf = d2f_fast(l * w);
+    l = ls_density(c.rho, sf::mul(w, A[0]), c.rmin, c.rmax);
+    at = d2f_fast(sf::mul(l, w));
   }
   *l_out = l;
-  if (ls_certified<DIM>(D, c, A, sf)) return true;
-  const double fb = ls_psi<DIM>(D, c.U0, A, l * w, c.smin);
-  *fb_out = fb;
-  if (fb >= 0.0) return true;
-  if (c.psi0 < 0.0) {
-    *l_out = 0.0;
-    return true;
-  }
-  return false;
+  return ls_certified<DIM>(D, c, A, at);
 }
 
 // Root of psi(t) on (0, l) in FP32, psi(0) = psi0 >= 0 > psi(l), t in units of P = w A: Newton steps from the
@@ -1008,20 +1005,21 @@ __device__ __forceinline__ bool line_search_head(const Dev& D, const LsRow<DIM>&
 template <int DIM>
 __device__ __forceinline__ float ls_root_f32(const Dev& D, const double* U0, const double* A, double w, double smin,
                                              double l, double psi0) {
-  const float P0 = (float)(w * A[0]), PE = (float)(w * A[DIM + 1]), r0 = (float)U0[0], ir0 = 1.f / r0;
+  // conversions on the integer pipe and products in FP32: this is a first approximation
+  const float wf = to_f32(w), P0 = wf * to_f32(A[0]), PE = wf * to_f32(A[DIM + 1]), r0 = to_f32(U0[0]), ir0 = 1.f / r0;
   float mP = 0.f, PP = 0.f, m0sq = 0.f;
 #pragma unroll
   for (int k = 0; k < DIM; ++k) {
-    const float m0 = (float)U0[1 + k], Pm = (float)(w * A[1 + k]);
+    const float m0 = to_f32(U0[1 + k]), Pm = wf * to_f32(A[1 + k]);
     mP = fmaf(m0, Pm, mP);
     PP = fmaf(Pm, Pm, PP);
     m0sq = fmaf(m0, m0, m0sq);
   }
   // s_min rho0^gamma = E0 - |m0|^2 / (2 rho0) - psi(0).  Sums of products are written as explicit fused
   // operations, so that every instantiation rounds alike.
-  const float psi0f = (float)psi0;
-  const float sg0 = fmaf(__fmul_rn(-0.5f, m0sq), ir0, (float)U0[DIM + 1]) - psi0f;
-  float t = (float)l;
+  const float psi0f = to_f32(psi0);
+  const float sg0 = fmaf(__fmul_rn(-0.5f, m0sq), ir0, to_f32(U0[DIM + 1])) - psi0f;
+  float t = to_f32(l);
 #pragma unroll 1
   for (int it = 0; it < 12; ++it) {
     const float a = __fmul_rn(t, P0), ir = 1.f / (r0 + a);
@@ -1042,10 +1040,11 @@ __device__ __forceinline__ float ls_root_f32(const Dev& D, const double* U0, con
 // or so.
 constexpr double kPsiRounding = 2.220446049250313e-16;
 
-// The search of an entry whose head found psi(l_rho) < 0 <= psi(0), from the same values.  Newton steps in
-// FP64 from the FP32 root reach the rounding of psi in two or three evaluations; every evaluated point
-// narrows the bracket [a, b] of feasible and infeasible ends.  The search ends where the step is at most
-// half the tolerance, or where psi or the bracket is below psi's own rounding (then its sign, not its
+// A queued search: l_rho from the density bounds in closed form; psi(l_rho) >= 0, and l_rho is the answer, or
+// psi(0) < 0 (roundoff), and 0 is; else a feasible point within ls_tol, or psi's rounding, of the root in between.
+// Newton steps in FP64 from the FP32 root reach the rounding of psi in two or three evaluations; every
+// evaluated point narrows the bracket [a, b] of feasible and infeasible ends.  The search ends where the step
+// is at most half the tolerance, or where psi or the bracket is below psi's own rounding (then its sign, not its
 // size, is all there is): at that point when it is feasible, else at one just before it that is.  A step that
 // leaves the bracket, or does not settle in a few, hands over to the plain bracketed iteration (chord
 // root, tangent root from the infeasible end, and a bisection where the bracket has not halved), which is
@@ -1059,79 +1058,72 @@ constexpr double kPsiRounding = 2.220446049250313e-16;
 // iteration: 110 -> 24 us for 1,435 searches (Q2, 33 x 47 quads), 1,207 -> 238 us for 493,000 (Q1,
 // 48 x 40 x 44 hexahedra), 316 -> 66 us for 91,000 (Q2, 1024^2).
 template <int DIM>
-__device__ __forceinline__ double line_search_tail(const Dev& D, const double* U0, const double* A, double w,
-                                                   double rmin, double rmax, double smin) {
-  enum { kZero, kNewton, kBack, kEnd, kChord, kTangent, kMiddle };
-  double l = 1.0;  // the density bounds in closed form, as in the head
-  {
-    const double Pr = __dmul_rn(w, A[0]);
-    if (U0[0] + Pr < rmin) l = (rmin - U0[0]) / Pr;
-    if (U0[0] + Pr > rmax) l = (rmax - U0[0]) / Pr;
-    if (!(l > 0.0)) l = 0.0;
-    if (l > 1.0) l = 1.0;
-  }
+__device__ __forceinline__ double line_search(const Dev& D, const double* U0, const double* A, double w, double rmin,
+                                              double rmax, double smin) {
+  enum { kFull, kZero, kNewton, kBack, kChord, kTangent, kMiddle };
+  // comparisons with the non-negative ends of the bracket, on the integer pipe
+  auto above = [](double x, double y) { return __double_as_longlong(x) > __double_as_longlong(y); };
+  const double l = ls_density(U0[0], sf::mul(w, A[0]), rmin, rmax);
   double a = 0.0, b = l, fa = 0.0, fb = 0.0, dfb = 0.0;
-  double t = 0.0, t0 = 0.0, back = 0.0, width = 0.0, tn = 0.0;
-  int phase = kZero, count = 0;
-  bool have_b = false;  // psi(b) and its slope are known
+  double t = l, t0 = 0.0, back = 0.0, width = 0.0, tn = 0.0;
+  int phase = kFull, count = 0;
   for (;;) {
     double d;
     const double f = ls_psi_dpsi<DIM>(D, U0, A, t * w, smin, &d);
     d *= w;
     const bool ok = f >= 0.0;
+    if (phase == kFull) {
+      if (ok) return l;
+      fb = f;
+      dfb = d;
+      t = 0.0;
+      phase = kZero;
+      continue;
+    }
     if (phase == kZero) {
       if (!ok) return 0.0;
       fa = f;
-      t = D.ls_maxit >= 8 ? (double)ls_root_f32<DIM>(D, U0, A, w, smin, l, f) : 0.0;
-      phase = kNewton;
-      if (t > a && t < b) continue;
-      phase = kEnd;
-      t = b;
-      continue;
-    }
-    if (phase == kEnd && ok) return b;
-    if (ok) {
-      a = t;
-      fa = f;
+      t = D.ls_maxit >= 8 ? to_f64(ls_root_f32<DIM>(D, U0, A, w, smin, l, f)) : 0.0;
+      if (above(t, a) && above(b, t)) {
+        phase = kNewton;
+        continue;
+      }
     } else {
-      b = t;
-      fb = f;
-      dfb = d;
-      have_b = true;
-    }
-    if (phase == kNewton && d < 0.0) {
-      const double id = 1.0 / d, step = __dmul_rn(f, id);
-      const double noise = -kPsiRounding * fma(t * w, A[DIM + 1], U0[DIM + 1]) * id;
-      if (b - a <= fmax(D.ls_tol, 4.0 * noise)) return a;
-      const double thr = fmax(0.5 * D.ls_tol, noise);
-      if (fabs(step) <= thr) {
+      if (ok) {
+        a = t;
+        fa = f;
+      } else {
+        b = t;
+        fb = f;
+        dfb = d;
+      }
+      if (phase == kNewton && d < 0.0) {
+        const double id = rcp64(d), step = __dmul_rn(f, id);
+        const double noise = abs_bits(__dmul_rn(kPsiRounding * id, fma(t * w, A[DIM + 1], U0[DIM + 1])));
+        if (!above(b - a, pmax(D.ls_tol, sf::mul_pow2(noise, 2)))) return a;
+        const double thr = pmax(sf::mul_pow2(D.ls_tol, -1), noise);
+        if (!above(abs_bits(step), thr)) {
+          if (ok) return t;
+          back = abs_bits(step) + thr;
+          t0 = t;
+          t = t0 - back;
+          if (!above(t, a)) return a;
+          phase = kBack;
+          count = 0;
+          continue;
+        }
+        t -= step;
+        if (above(t, a) && above(b, t) && ++count < 8) continue;
+      }
+      if (phase == kBack) {
         if (ok) return t;
-        back = fabs(step) + thr;
-        t0 = t;
+        back = sf::mul_pow2(back, 2);
         t = t0 - back;
-        if (!(t > a)) return a;
-        phase = kBack;
-        count = 0;
-        continue;
-      }
-      t -= step;
-      if (t > a && t < b && ++count < 8) continue;
-    }
-    if (phase == kBack) {
-      if (ok) return t;
-      back *= 4.0;
-      t = t0 - back;
-      if (!(t > a)) return a;  // the bracket is no wider than what the step and the rounding leave open
-      if (++count < 3) continue;
-    }
-    if (phase <= kBack) {  // the Newton steps did not settle: on to the plain iteration
-      phase = kEnd;
-      if (!have_b) {
-        t = b;
-        continue;
+        if (!above(t, a)) return a;  // the bracket is no wider than what the step and the rounding leave open
+        if (++count < 3) continue;
       }
     }
-    if (phase == kEnd) {
+    if (phase <= kBack) {  // the Newton steps did not settle, or there is no start for them: the plain iteration
       count = 0;
       phase = kMiddle;
       width = 2.0 * (b - a);  // (the bisection below is for an iteration that has been run)
@@ -1168,12 +1160,16 @@ __device__ __forceinline__ double line_search_tail(const Dev& D, const double* U
   }
 }
 
-// The searches that need the tail are rare (well under 1% of the entries) but take ~10 iterations, and a
-// lane that iterates holds up its whole warp; the sweep kernels therefore queue them (entry, row) and
-// k_lsfix runs the tails with every lane busy.  Queue item: x = CSR entry e, or -(b + 1) for boundary
-// entry b; y = row i.
+// The searches that FP32 does not settle are few, and a lane that iterates holds up its whole warp; the sweep
+// kernels therefore queue them (entry, row) and k_lsfix runs them with every lane busy.  Queue item: x = CSR
+// entry e, or -(b + 1) for boundary entry b; y = row i.  One addition to the queue's length for the lanes that
+// come here together.
 __device__ __forceinline__ void ls_defer(const Scratch& S, int pass, int code, int i) {
-  const unsigned k = atomicAdd(S.lsq_n + pass, 1u);
+  const unsigned m = __activemask(), lane = threadIdx.x & 31u;
+  const int leader = __ffs((int)m) - 1;
+  unsigned k = 0;
+  if ((int)lane == leader) k = atomicAdd(S.lsq_n + pass, (unsigned)__popc(m));
+  k = __shfl_sync(m, k, leader) + (unsigned)__popc(m & ((1u << lane) - 1u));
   S.lsq[k] = make_int2(code, i);
 }
 

@@ -357,8 +357,8 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
       S.l1[e] = 1.0;
       continue;
     }
-    double l, fb;
-    if (line_search_head<DIM>(D, ls, A, ikm, ikmf, &l, &fb))
+    double l;
+    if (line_search_sure<DIM>(D, ls, A, ikm, ikmf, &l))
       S.l1[e] = l;
     else
       ls_defer(S, 0, e, i);
@@ -367,8 +367,8 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
     double A[M];
 #pragma unroll
     for (int q = 0; q < M; ++q) A[q] = S.AB[(size_t)q * D.nb + b];
-    double l, fb;
-    if (line_search_head<DIM>(D, ls, A, ikm, ikmf, &l, &fb))
+    double l;
+    if (line_search_sure<DIM>(D, ls, A, ikm, ikmf, &l))
       S.l1B[b] = l;
     else
       ls_defer(S, 0, -(b + 1), i);

@@ -69,8 +69,8 @@ __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last
     double A[M];
 #pragma unroll
     for (int q = 0; q < M; ++q) A[q] = S.A[q * nnz + e];
-    double l, fb;
-    if (line_search_head<DIM>(D, ls, A, w, d2f_fast(w), &l, &fb))
+    double l;
+    if (line_search_sure<DIM>(D, ls, A, w, d2f_fast(w), &l))
       S.l2[e] = l;
     else
       ls_defer(S, 1, e, i);
@@ -81,8 +81,8 @@ __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last
     double A[M];
 #pragma unroll
     for (int q = 0; q < M; ++q) A[q] = S.AB[q * nb + b];
-    double l, fb;
-    if (line_search_head<DIM>(D, ls, A, w, d2f_fast(w), &l, &fb))
+    double l;
+    if (line_search_sure<DIM>(D, ls, A, w, d2f_fast(w), &l))
       S.l2B[b] = l;
     else
       ls_defer(S, 1, -(b + 1), i);
@@ -97,13 +97,14 @@ __global__ void __maxnreg__(72) k_limit2(Src src, int sliced, int last) {
 
 // The deferred line searches of one limiter pass (pass 0: from U^L with P = A / (kappa_i m_i), written to
 // l1; pass 1: from U^(1) with P = (1 - l1_ij) A / (kappa_i m_i), written to l2).  One thread per queued
-// entry, grid-stride over the queue.
+// entry, grid-stride over the queue, the warps numbered through the blocks first: a short queue then has one warp
+// on each of many SMs instead of four on a few, where they would share the FP64 pipe.
 template <int DIM, class Src>
 __device__ __forceinline__ void lsfix_body(const Src& src, int pass) {
   constexpr int M = DIM + 2;
   __shared__ Ctx sctx;
   int lb, blocks_per_inst;
-  if ((unsigned)src.queue_length(pass, &lb) <= (unsigned)lb * blockDim.x) return;  // a block with no item
+  if ((unsigned)src.queue_length(pass, &lb) <= (unsigned)lb * 32u) return;  // a block with no item
   const Ctx& c = src.get(&sctx, &lb, &blocks_per_inst);
   if (finished(c)) return;
   const Dev& D = c.D;
@@ -111,7 +112,8 @@ __device__ __forceinline__ void lsfix_body(const Src& src, int pass) {
   const unsigned count = S.lsq_n[pass];
   const size_t n = D.n, nnz = D.nnz, nb = D.nb;
   const unsigned stride = (unsigned)blocks_per_inst * blockDim.x;
-  for (unsigned k = lb * blockDim.x + threadIdx.x; k < count; k += stride) {
+  const unsigned first = ((threadIdx.x >> 5) * (unsigned)blocks_per_inst + (unsigned)lb) * 32u + (threadIdx.x & 31u);
+  for (unsigned k = first; k < count; k += stride) {
     const int2 it = S.lsq[k];
     const int i = it.y;
     const bool bnd = it.x < 0;
@@ -125,7 +127,7 @@ __device__ __forceinline__ void lsfix_body(const Src& src, int pass) {
     }
     double w = D.inv_km[i];
     if (pass == 1) w = (1.0 - (bnd ? S.l1B[e] : pmin(S.l1[e], S.l1[D.tr[e]]))) * w;
-    const double l = line_search_tail<DIM>(D, U0, A, w, S.bounds[i], S.bounds[n + i], S.bounds[2 * n + i]);
+    const double l = line_search<DIM>(D, U0, A, w, S.bounds[i], S.bounds[n + i], S.bounds[2 * n + i]);
     double* dst = pass == 0 ? (bnd ? S.l1B : S.l1) : (bnd ? S.l2B : S.l2);
     dst[e] = l;
   }
