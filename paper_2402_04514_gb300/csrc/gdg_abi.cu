@@ -147,6 +147,18 @@ EllLayout ell_layout(int64_t n, int nl, Len len) {
 
 int64_t padded_elements(int64_t nel) { return (nel + gdg::kEll - 1) / gdg::kEll * gdg::kEll; }
 
+// The slot of node i (gdg::Node), and a per-node array in the order of the slots, zero where there is no node.
+int64_t node_slot(int64_t i, int nl) {
+  const int64_t E = i / nl;
+  return ((E / gdg::kEll) * nl + i % nl) * gdg::kEll + E % gdg::kEll;
+}
+template <class T>
+std::vector<T> by_slot(const std::vector<T>& a, int nl, int64_t ns) {
+  std::vector<T> r((size_t)ns, T(0));
+  for (int64_t i = 0; i < (int64_t)a.size(); ++i) r[(size_t)node_slot(i, nl)] = a[(size_t)i];
+  return r;
+}
+
 Layout make_layout(int dim, int64_t n, int64_t nnz, int64_t nb, int nl, int64_t ne, int64_t nel) {
   const int64_t m = dim + 2;
   Layout Lo;
@@ -196,12 +208,16 @@ int param_arrays(const gdg_handle* h, const gdg_params& p, ParamArrays& A) {
 }
 
 int upload_param_arrays(gdg_handle* h, const ParamArrays& A) {
-  const int64_t n = h->n, nnz = h->nnz_ell;
+  const int64_t ns = h->ns, nnz = h->nnz_ell;
+  const int nl = h->n_loc;
   cudaError_t e;
   if ((nnz > 0 && (e = cudaMemcpy(h->d_mu, A.mu.data(), sizeof(double) * nnz, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (n > 0 && (e = cudaMemcpy(h->d_rminus, A.rm.data(), sizeof(double) * n, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (n > 0 && (e = cudaMemcpy(h->d_rplus, A.rp.data(), sizeof(double) * n, cudaMemcpyHostToDevice)) != cudaSuccess) ||
-      (n > 0 && (e = cudaMemcpy(h->d_muB, A.muB.data(), sizeof(double) * n, cudaMemcpyHostToDevice)) != cudaSuccess))
+      (ns > 0 &&
+       (e = cudaMemcpy(h->d_rminus, by_slot(A.rm, nl, ns).data(), sizeof(double) * ns, cudaMemcpyHostToDevice)) != cudaSuccess) ||
+      (ns > 0 &&
+       (e = cudaMemcpy(h->d_rplus, by_slot(A.rp, nl, ns).data(), sizeof(double) * ns, cudaMemcpyHostToDevice)) != cudaSuccess) ||
+      (ns > 0 &&
+       (e = cudaMemcpy(h->d_muB, by_slot(A.muB, nl, ns).data(), sizeof(double) * ns, cudaMemcpyHostToDevice)) != cudaSuccess))
     return cuda_fail(e);
   const gdg_params& p = h->params;
   Dev& D = h->D;
@@ -279,6 +295,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   h->degree = P->degree;
   h->n_loc = nl;
   h->n = n;
+  h->ns = padded_elements(n / nl) * nl;
   h->nnz = nnz;
   h->nb = nb;
   h->gamma = P->gamma;
@@ -387,7 +404,6 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   std::vector<int> b_ptr(n + 1, 0);
   for (int64_t b = 0; b < nb; ++b) b_ptr[P->b_node[b] + 1]++;
   for (int64_t i = 0; i < n; ++i) b_ptr[i + 1] += b_ptr[i];
-  h->borig = border;
   // partition of unity (Lemma LemPart)
   {
     std::vector<char> bad(n, 0);
@@ -478,7 +494,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   parallel_for(nnz, [&](int64_t b, int64_t e) {
     for (int64_t q = b; q < e; ++q) {
       const int64_t pq = h->epos[q];
-      col_e[pq] = h->col[q];
+      col_e[pq] = (int)node_slot(h->col[q], nl);
       tr_e[pq] = h->epos[h->tr[q]];
       cnorm_e[pq] = cnorm[q];
       mij_e[pq] = mij[q];
@@ -513,9 +529,16 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   std::vector<int> edge_e(edges.size()), edge_i(edges.size());
   for (size_t k = 0; k < edges.size(); ++k) {
     edge_e[k] = edges[k].first;
-    edge_i[k] = edges[k].second;
+    edge_i[k] = (int)node_slot(edges[k].second, nl);
   }
   const int64_t ne = (int64_t)edge_e.size();
+  // the boundary entries in the order of their nodes' slots, the caller's order within a node
+  std::stable_sort(border.begin(), border.end(),
+                   [&](int a, int b) { return node_slot(P->b_node[a], nl) < node_slot(P->b_node[b], nl); });
+  h->borig = border;
+  std::vector<int> b_slot(h->ns + 1, 0);
+  for (int64_t b = 0; b < nb; ++b) b_slot[node_slot(P->b_node[b], nl) + 1]++;
+  for (int64_t t = 0; t < h->ns; ++t) b_slot[t + 1] += b_slot[t];
   std::vector<double> bnorm(nb), bn((size_t)dim * nb);
   std::vector<int> btype(nb), bnode(nb);
   for (int64_t t = 0; t < nb; ++t) {
@@ -525,14 +548,15 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
     bnorm[t] = std::sqrt(c2);
     for (int k = 0; k < dim; ++k) bn[(size_t)k * nb + t] = P->b_c[(size_t)k * nb + b] / bnorm[t];
     btype[t] = P->b_type[b];
-    bnode[t] = P->b_node[b];
+    bnode[t] = (int)node_slot(P->b_node[b], nl);
   }
 
   ParamArrays pa;
   if (int rc = param_arrays(h, h->params, pa); rc != GDG_OK) return fail(rc);
 
   // ---- device arena ----
-  const Layout Lo = make_layout(dim, n, NE, nb, nl, ne, nel_pad);
+  const int64_t ns = h->ns;
+  const Layout Lo = make_layout(dim, ns, NE, nb, nl, ne, nel_pad);
 #define GDG_F(name, T, cnt) const size_t o_##name = Lo.o_##name;
   GDG_ARENA(GDG_F)
 #undef GDG_F
@@ -551,25 +575,25 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
     if (bytes == 0) return cudaSuccess;
     return cudaMemcpy(ptr(o), src, bytes, cudaMemcpyHostToDevice);
   };
-  if ((ce = up(o_rbeg, rbeg.data(), sizeof(int) * n)) != cudaSuccess ||
-      (ce = up(o_rend, rend.data(), sizeof(int) * n)) != cudaSuccess ||
-      (ce = up(o_sten, sten_ell.data(), sizeof(int) * n)) != cudaSuccess ||
+  if ((ce = up(o_rbeg, by_slot(rbeg, nl, ns).data(), sizeof(int) * ns)) != cudaSuccess ||
+      (ce = up(o_rend, by_slot(rend, nl, ns).data(), sizeof(int) * ns)) != cudaSuccess ||
+      (ce = up(o_sten, by_slot(sten_ell, nl, ns).data(), sizeof(int) * ns)) != cudaSuccess ||
       (ce = up(o_col, col_e.data(), sizeof(int) * NE)) != cudaSuccess ||
       (ce = up(o_tr, tr_e.data(), sizeof(int) * NE)) != cudaSuccess ||
       (ce = up(o_cnorm, cnorm_e.data(), sizeof(double) * NE)) != cudaSuccess ||
       (ce = up(o_cn, cn_e.data(), sizeof(double) * dim * NE)) != cudaSuccess ||
       (ce = up(o_mij, mij_e.data(), sizeof(double) * NE)) != cudaSuccess ||
-      (ce = up(o_mi, h->mi.data(), sizeof(double) * n)) != cudaSuccess ||
-      (ce = up(o_imi, inv_mi.data(), sizeof(double) * n)) != cudaSuccess ||
-      (ce = up(o_ikm, inv_km.data(), sizeof(double) * n)) != cudaSuccess ||
-      (ce = up(o_bptr, b_ptr.data(), sizeof(int) * (n + 1))) != cudaSuccess ||
+      (ce = up(o_mi, by_slot(h->mi, nl, ns).data(), sizeof(double) * ns)) != cudaSuccess ||
+      (ce = up(o_imi, by_slot(inv_mi, nl, ns).data(), sizeof(double) * ns)) != cudaSuccess ||
+      (ce = up(o_ikm, by_slot(inv_km, nl, ns).data(), sizeof(double) * ns)) != cudaSuccess ||
+      (ce = up(o_bptr, b_slot.data(), sizeof(int) * (ns + 1))) != cudaSuccess ||
       (ce = up(o_bnorm, bnorm.data(), sizeof(double) * nb)) != cudaSuccess ||
       (ce = up(o_bn, bn.data(), sizeof(double) * dim * nb)) != cudaSuccess ||
       (ce = up(o_btype, btype.data(), sizeof(int) * nb)) != cudaSuccess ||
       (ce = up(o_borig, border.data(), sizeof(int) * nb)) != cudaSuccess ||
       (ce = up(o_bnode, bnode.data(), sizeof(int) * nb)) != cudaSuccess ||
       (ce = up(o_minv, minv_g.data(), sizeof(sf::fixp) * minv_g.size())) != cudaSuccess ||
-      (ce = up(o_wexp, wexp.data(), sizeof(int) * n)) != cudaSuccess ||
+      (ce = up(o_wexp, by_slot(wexp, nl, ns).data(), sizeof(int) * ns)) != cudaSuccess ||
       (ce = up(o_ee, edge_e.data(), sizeof(int) * ne)) != cudaSuccess ||
       (ce = up(o_ei, edge_i.data(), sizeof(int) * ne)) != cudaSuccess ||
       (ce = cudaMemset(ptr(o_flags), 0, 16)) != cudaSuccess)
@@ -577,6 +601,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
 
   Dev& D = h->D;
   D.n = (int)n;
+  D.ns = (int)ns;
   D.nnz = (int)NE;
   D.nb = (int)nb;
   D.n_loc = nl;
@@ -638,6 +663,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   S.l2 = (double*)ptr(o_l2);
   S.l2B = (double*)ptr(o_l2B);
   S.U1 = (double*)ptr(o_U1);
+  S.Us = S.U1;
   S.rem = (unsigned char*)ptr(o_rem);
   S.flags = (unsigned*)ptr(o_flags);
   S.lsq_n = S.flags + 2;
@@ -672,7 +698,8 @@ int gdg_footprint(const gdg_problem* P, int64_t* bytes) {
     }
   if (P->n % P->n_loc != 0) return GDG_EINVAL;
   const EllLayout EL = ell_layout(P->n, P->n_loc, [&](int64_t i) { return P->row_ptr[i + 1] - P->row_ptr[i]; });
-  *bytes = (int64_t)make_layout(P->dim, P->n, EL.total, P->nb, P->n_loc, ne, padded_elements(P->n / P->n_loc)).total;
+  *bytes = (int64_t)make_layout(P->dim, padded_elements(P->n / P->n_loc) * P->n_loc, EL.total, P->nb, P->n_loc, ne,
+                                padded_elements(P->n / P->n_loc)).total;
   return GDG_OK;
 }
 
@@ -1002,17 +1029,17 @@ int gdg_debug_export(gdg_handle* h, const char* name, double* dst, int64_t count
   const double* src = nullptr;
   int64_t want = -1;
   int kind = 0;  // 0 plain copy, 1 symmetrised per-entry limiter, 2 boundary order
-  bool per_entry = false;
+  bool per_entry = false, per_node = false;
   std::string nm(name);
   if (nm == "dL") { src = h->S.dL; want = nnz; per_entry = true; }
   else if (nm == "dB") { src = h->S.dB; want = nb; kind = 2; }
-  else if (nm == "N") { src = h->S.N; want = n; }
-  else if (nm == "UL") { src = h->S.UL; want = m * n; }
-  else if (nm == "U1") { src = h->S.U1; want = m * n; }
+  else if (nm == "N") { src = h->S.N; want = n; per_node = true; }
+  else if (nm == "UL") { src = h->S.UL; want = m * n; per_node = true; }
+  else if (nm == "U1") { src = h->S.U1; want = m * n; per_node = true; }
   else if (nm == "A") { src = h->S.A; want = m * nnz; per_entry = true; }
-  else if (nm == "rho_min") { src = h->S.bounds; want = n; }
-  else if (nm == "rho_max") { src = h->S.bounds + n; want = n; }
-  else if (nm == "s_min") { src = h->S.bounds + 2 * n; want = n; }
+  else if (nm == "rho_min") { src = h->S.bounds; want = n; per_node = true; }
+  else if (nm == "rho_max") { src = h->S.bounds + h->ns; want = n; per_node = true; }
+  else if (nm == "s_min") { src = h->S.bounds + 2 * h->ns; want = n; per_node = true; }
   else if (nm == "l1") { src = h->S.l1; want = nnz; kind = 1; }
   else if (nm == "l2") { src = h->S.l2; want = nnz; kind = 1; }
   else if (nm == "ls_deferred") { want = 2; kind = 3; }
@@ -1027,8 +1054,10 @@ int gdg_debug_export(gdg_handle* h, const char* name, double* dst, int64_t count
     dst[1] = q[1];
     return GDG_OK;
   }
-  // per-entry arrays live in sliced-ELL order on the device (their length NE per component)
-  const int64_t dev_count = (per_entry || kind == 1) ? want / std::max<int64_t>(nnz, 1) * NE : want;
+  // per-entry arrays live in sliced-ELL order on the device (their length NE per component), per-node ones by slots
+  const int64_t dev_count = (per_entry || kind == 1) ? want / std::max<int64_t>(nnz, 1) * NE
+                            : per_node               ? want / std::max<int64_t>(n, 1) * h->ns
+                                                     : want;
   std::vector<double> tmp(dev_count);
   if (dev_count > 0 &&
       (e = cudaMemcpy(tmp.data(), src, sizeof(double) * dev_count, cudaMemcpyDeviceToHost)) != cudaSuccess)
@@ -1037,16 +1066,17 @@ int gdg_debug_export(gdg_handle* h, const char* name, double* dst, int64_t count
     for (int64_t r = 0; r < want / std::max<int64_t>(nnz, 1); ++r)
       for (int64_t q = 0; q < nnz; ++q) dst[r * nnz + h->eorig[q]] = tmp[r * NE + h->epos[q]];
     if (nm == "A" && h->D.order == GDG_ORDER_LIMITED && h->D.passes > 0) {  // rows whose A is zero are not stored
-      std::vector<unsigned char> rem(n);
-      if (n > 0 && (e = cudaMemcpy(rem.data(), h->S.rem, n, cudaMemcpyDeviceToHost)) != cudaSuccess)
+      std::vector<unsigned char> rem(h->ns);
+      if (n > 0 && (e = cudaMemcpy(rem.data(), h->S.rem, h->ns, cudaMemcpyDeviceToHost)) != cudaSuccess)
         return cuda_fail(e);
       for (int64_t i = 0; i < n; ++i)
-        if (rem[i] == 2)
+        if (rem[node_slot(i, h->n_loc)] == 2)
           for (int64_t q = h->row_ptr[i]; q < h->row_ptr[i + 1]; ++q)
             for (int64_t r = 0; r < m; ++r) dst[r * nnz + h->eorig[q]] = 0.0;
     }
-  } else if (kind == 0) {
-    std::memcpy(dst, tmp.data(), sizeof(double) * want);
+  } else if (per_node) {
+    for (int64_t r = 0; r < want / std::max<int64_t>(n, 1); ++r)
+      for (int64_t i = 0; i < n; ++i) dst[r * n + i] = tmp[r * h->ns + node_slot(i, h->n_loc)];
   } else if (kind == 1) {
     for (int64_t q = 0; q < want; ++q) dst[h->eorig[q]] = std::min(tmp[h->epos[q]], tmp[h->epos[h->tr[q]]]);
   } else {

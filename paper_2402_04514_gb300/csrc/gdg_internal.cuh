@@ -30,17 +30,19 @@ __host__ __device__ inline RootQ root_q(int q) { return RootQ{sf::root_const(q),
 constexpr int kEll = 32;
 
 // Everything a kernel needs, passed by value.  Per-entry arrays are device pointers in the sliced-ELL
-// order above (row i's entries at rbeg[i], rbeg[i] + kEll, ... below rend[i]); per-node arrays in node
-// order (rows element-contiguous); boundary entries are sorted by node (b_ptr indexes them).
+// order above (row i's entries at rbeg[i], rbeg[i] + kEll, ... below rend[i]); per-node arrays in the order of the
+// slots (Node below), which also number the nodes in col, edge_i and bnode; boundary entries are sorted by
+// slot (b_ptr indexes them).
 struct Dev {
   int n, nnz, nb, n_loc;      // nnz: the length of the per-entry arrays, padding included
+  int ns;                     // slots: n_loc times the elements in whole ELL groups
   int nel;                    // elements (n / n_loc)
   unsigned long long nl_mul;  // floor(x / n_loc) = (x * nl_mul) >> nl_shift for 0 <= x < 2^31 (div_nl)
   int nl_shift;
   // rows
-  const int* rbeg;      // [n] position of row i's first entry
-  const int* rend;      // [n] end of row i: rbeg[i] + kEll * (row length)
-  const int* sten_end;  // [n] end of row i's stencil entries: I(i) is rbeg[i], rbeg[i] + kEll, ... below it
+  const int* rbeg;      // [ns] position of row i's first entry
+  const int* rend;      // [ns] end of row i: rbeg[i] + kEll * (row length)
+  const int* sten_end;  // [ns] end of row i's stencil entries: I(i) is rbeg[i], rbeg[i] + kEll, ... below it
   const int* col;       // [nnz]
   const int* tr;        // [nnz] position of the transposed entry (j, i)
   const double* cnorm;  // [nnz] |c_ij| (0 when c_ij = 0)
@@ -48,13 +50,13 @@ struct Dev {
   const double* mij;    // [nnz] consistent mass m_ij (0 across elements)
   const double* mu;     // [nnz] c_k h_ij^{p_k} for collocated pairs, else 0 (Sec. 5.1, eq. (ViscMin))
   // nodes
-  const double* mi;     // [n]
-  const double* inv_mi; // [n]
-  const double* inv_km; // [n] 1 / (kappa_i m_i), Sec. 5.4, eq. (ConvexScheme)
-  const double* rminus; // [n] r_h^- (Sec. 5.4)
-  const double* rplus;  // [n] r_h^+
-  const double* muB;    // [n] c_k h_i^{p_k} (boundary minimal-viscosity factor)
-  const int* b_ptr;     // [n+1]
+  const double* mi;     // [ns]
+  const double* inv_mi; // [ns]
+  const double* inv_km; // [ns] 1 / (kappa_i m_i), Sec. 5.4, eq. (ConvexScheme)
+  const double* rminus; // [ns] r_h^- (Sec. 5.4)
+  const double* rplus;  // [ns] r_h^+
+  const double* muB;    // [ns] c_k h_i^{p_k} (boundary minimal-viscosity factor)
+  const int* b_ptr;     // [ns + 1]
   // boundary entries (sorted by node)
   const double* bnorm;  // [nb] |c_i^{d,k}|
   const double* bn;     // [dim][nb] unit normals
@@ -62,7 +64,7 @@ struct Dev {
   const int* borig;     // [nb] index of the entry in the caller's order (for Dirichlet data)
   const int* bnode;     // [nb] node of the entry
   const int2* MKinv;    // [n / n_loc][n_loc][n_loc] rows of M_K^{-1} in fixed point (sf::fixp)
-  const int* wexp;      // [n] exponent field of the largest entry of each row
+  const int* wexp;      // [ns] exponent field of the largest entry of each row
   // canonical stencil edges: entries (i, j) with c_ij != 0 and i < j, in entry order
   int ne;
   const int* edge_e;    // [ne] entry index of (i, j)
@@ -101,13 +103,27 @@ __device__ __forceinline__ int div_nl(const Dev& D, int x) {
   return (int)(((unsigned long long)(unsigned)x * D.nl_mul) >> D.nl_shift);
 }
 
-// The row of slot t of a one-thread-per-row kernel (row_slots below), -1 past the mesh.
-__device__ __forceinline__ int row_node(const Dev& D, int t, int sliced) {
-  if (!sliced) return t < D.n ? t : -1;
+// A node: its number i in the caller's arrays (-1 past the mesh) and its slot t in the library's own.  The library's
+// arrays hold the nodes in the order of the ELL slices: slot (g n_loc + l) kEll + lane is local index l of element
+// g kEll + lane, so that a warp, which takes one local index of consecutive elements, reads and writes them
+// contiguously, its own nodes as well as their neighbours.  In the caller's order its lanes were n_loc apart and took
+// a sector each.  In us per launch at Q3 96^2: k_edge 65 -> 52, k_high 155 -> 133, k_low 62 -> 56; at Q2 1024^2 k_low 968 ->
+// 845, k_high 1,449 -> 1,384, k_limit2 471 -> 422; k_prim, which now also copies the state, 444 -> 454.
+struct Node {
+  int i, t;
+};
+__device__ __forceinline__ Node node_of_slot(const Dev& D, int t) {
   const int sl = t / kEll;
   const int g = div_nl(D, sl);
   const int E = g * kEll + (t & (kEll - 1));
-  return E < D.nel ? E * D.n_loc + (sl - g * D.n_loc) : -1;
+  return Node{E < D.nel ? E * D.n_loc + (sl - g * D.n_loc) : -1, t};
+}
+// The row of thread x of a one-thread-per-row kernel (row_slots below), by slots or by the caller's numbers.
+__device__ __forceinline__ Node row_node(const Dev& D, int x, int sliced) {
+  if (sliced) return node_of_slot(D, x);
+  if (x >= D.n) return Node{-1, 0};
+  const int E = div_nl(D, x);
+  return Node{x, ((E / kEll) * D.n_loc + (x - E * D.n_loc)) * kEll + (E & (kEll - 1))};
 }
 
 // Equation-of-state constants of Dev for gamma (host side; gdg_setup and the wave-speed check).
@@ -144,7 +160,7 @@ inline void set_eos(Dev& D, double gamma) {
 }
 
 struct Scratch {
-  double* prim;    // [NPRIM][n]
+  double* prim;    // [NPRIM][ns]
   double* dL;      // [nnz]
   double* G;       // [m][nnz] (f(U_j) - f(U_i)) c_ij of stencil entries (from the edge sweep; symmetric in i, j)
   double* psi;     // [nnz] (m_j . c_ij)(f_j - f_i), the indicator's term of the entry (mixed: m_j . c_ij)
@@ -155,19 +171,20 @@ struct Scratch {
   double* UB;      // [m][nb] boundary states U_i^{d,k}
   double* gB;      // [m][nb] f(U_i^{d,k}) c_i^{d,k}
   double* gI;      // [m][nb] f(U_i) c_i^{d,k}
-  double* UL;      // [m][n]
-  double* RHSL;    // [m][n] low-order right-hand side (sum of fluxes and viscous terms)
-  double* N;       // [n]
-  double* agg;     // [3][n] one-hop aggregates (rho min, rho max, s~ min)
+  double* UL;      // [m][ns]
+  double* RHSL;    // [m][ns] low-order right-hand side (sum of fluxes and viscous terms)
+  double* N;       // [ns]
+  double* agg;     // [3][ns] one-hop aggregates (rho min, rho max, s~ min)
   double* A;       // [m][nnz]
   double* AB;      // [m][nb]
-  double* bounds;  // [3][n] rho_min, rho_max, s~_min
+  double* bounds;  // [3][ns] rho_min, rho_max, s~_min
   double* l1;      // [nnz] per-row limiter coefficients, pass 1 (before symmetrisation)
   double* l1B;     // [nb]
   double* l2;      // [nnz] pass 2
   double* l2B;     // [nb]
-  double* U1;      // [m][n]
-  unsigned char* rem;  // [n] from the element sweep: 2 where all of row i's A is zero and therefore not stored; then from
+  double* U1;      // [m][ns]
+  double* Us;      // [m][ns] the stage input by slots, from k_prim to k_high (in the place of U1, which comes later)
+  unsigned char* rem;  // [ns] from the element sweep: 2 where all of row i's A is zero and therefore not stored; then from
                        // sweep C also 1 where the row has a pass-2 remainder (a symmetrised pass-1 factor below 1)
   unsigned int* flags;
   unsigned int* lsq_n;  // [2] lengths of the deferred line-search queues of passes 1 and 2
@@ -334,7 +351,7 @@ inline Sched default_sched() {
 // lane t % kEll of slice t / kEll = g n_loc + l, the row of local index l of element g kEll + t % kEll, so
 // that a warp's per-entry loads are contiguous (the nodes' own arrays are then read n_loc apart).
 __host__ __device__ inline long long row_slots(const Dev& D, bool sliced) {
-  return sliced ? (long long)((D.nel + kEll - 1) / kEll) * kEll * D.n_loc : (long long)D.n;
+  return sliced ? (long long)D.ns : (long long)D.n;
 }
 // Elements per block of the element sweep: the largest power of two <= kEll whose nodes fit the cap (so
 // that a block is an aligned part of one ELL group), at least one.
@@ -349,10 +366,12 @@ __host__ __device__ inline int high_threads(int n_loc, int eb) { return (eb * n_
 // entries are the longer chain, so they start first (as the last blocks they held up the end of the
 // launch: 291 against 245 us at Q2 301 x 259 with open sides).
 __host__ __device__ inline unsigned boundary_slots(int nb) { return ((unsigned)nb + 31u) & ~31u; }
+inline long long kernel_slots(int k, const Dev& D, const Sched& sc) {  // threads with work of a kernel shaped by bt
+  if (k == KN_MAXDT || k == KN_EDGE) return (long long)boundary_slots(D.nb) + D.ne;
+  return row_slots(D, k == KN_PRIM || ((sc.slices >> k) & 1));
+}
 inline long long kernel_blocks(int k, const Dev& D, const Sched& sc) {
   switch (k) {
-    case KN_MAXDT:
-    case KN_EDGE: return ((long long)boundary_slots(D.nb) + D.ne + sc.bt[k] - 1) / sc.bt[k];
     case KN_HIGH: {  // the groups of kEll elements, each in kEll / eb blocks
       const int eb = high_elems_per_block(D.n_loc, sc.high_cap);
       return eb > 0 ? ((long long)D.nel + kEll - 1) / kEll * (kEll / eb) : 0;
@@ -367,7 +386,7 @@ inline long long kernel_blocks(int k, const Dev& D, const Sched& sc) {
       const long long cover = D.n == 0 ? 0 : ((long long)D.nnz + D.nb + per_block - 1) / per_block;
       return cover < kLsfixMaxBlocks ? cover : kLsfixMaxBlocks;
     }
-    default: return (row_slots(D, (sc.slices >> k) & 1) + sc.bt[k] - 1) / sc.bt[k];
+    default: return (kernel_slots(k, D, sc) + sc.bt[k] - 1) / sc.bt[k];
   }
 }
 

@@ -10,6 +10,7 @@ struct gdg_handle {
   int device = 0;
   int dim = 0, degree = 0, n_loc = 0;
   int64_t n = 0, nnz = 0, nb = 0;
+  int64_t ns = 0;  // nodes in whole ELL groups: the length of the per-node arrays (gdg::Node)
   double gamma = 1.4, omega = 1.0;
   gdg_params params{};
   bool has_dirichlet = false;

@@ -18,8 +18,9 @@ constexpr int kMaxLocal = 32;  // n_loc limit of gdg_setup
 // element e0 + t % eb, so the lanes of a warp hold one local index of consecutive elements: rows of one
 // shape (equal trip counts through the row loops) whose entries lie side by side in the ELL slices.
 struct ElemSlot {
-  int i;      // the node, valid only if ok
+  int i, t;   // the node and its slot, valid only if ok
   int el, l;  // the element's place in the block and the node's local index
+  int g;      // the ELL group
   bool ok;
 };
 __device__ __forceinline__ ElemSlot element_slot(const Dev& D, int lb, int eb) {
@@ -32,6 +33,8 @@ __device__ __forceinline__ ElemSlot element_slot(const Dev& D, int lb, int eb) {
   const int E = g * kEll + (lb - g * per_group) * eb + r.el;
   r.ok = r.l < D.n_loc && E < D.nel;
   r.i = E * D.n_loc + r.l;
+  r.t = (g * D.n_loc + r.l) * kEll + (E & (kEll - 1));
+  r.g = g;
   return r;
 }
 
@@ -64,16 +67,16 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   if (finished(c)) return;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const double* U = c.U;
+  const double* U = S.Us;
   const ElemSlot es = element_slot(D, lb, eb);
-  const int i = es.i;
+  const int i = es.t;
   const bool valid = es.ok;
   // the shared arrays space elements n_loc + 1 apart for even n_loc: the lanes of a warp read one node of
   // each of consecutive elements, and an even stride would put pairs of them in the same bank
   const int stride_sh = D.n_loc + !(D.n_loc & 1);
   const int t0 = es.el * stride_sh;  // the element's first slot in the shared arrays
   const int sh = t0 + es.l;
-  const size_t n = D.n;
+  const size_t n = D.ns;
   const double tau = stage_tau(c);
   for (int k = threadIdx.x; k < M * kEll; k += blockDim.x) (&sE[0][0])[k] = 0;
   __syncthreads();
@@ -86,7 +89,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   bool quiet = true;                           // no viscous part of A in the row, and no boundary entry
   unsigned zeros = 0;                          // the stencil entries (of the row's first 32) without a viscous part
   if (valid) {
-    load_state<DIM>(U, D.n, i, Ui);
+    load_state<DIM>(U, D.ns, i, Ui);
     Ni = abs_bits(S.N[i]);
 #pragma unroll
     for (int q = 0; q < M; ++q) {
@@ -218,10 +221,9 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   }
   if (valid) {
     const int nl = D.n_loc;
-    const int ei = div_nl(D, i);
     // row il of the element's M_K^{-1}, stored grouped like the entries: (E, a, b) at
     // ((E / kEll * n_loc + a) * n_loc + b) * kEll + E % kEll
-    const int2* Minv = D.MKinv + ((size_t)(ei / kEll) * nl + es.l) * nl * kEll + (ei % kEll);
+    const int2* Minv = D.MKinv + ((size_t)es.g * nl + es.l) * nl * kEll + (i & (kEll - 1));
     const int we = D.wexp[i];
     if (flat) {
 #pragma unroll
@@ -270,7 +272,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
           du = to_f64(dUi[q]);
         else
           du = dUi[q];
-        store_out(c, (size_t)q * n + i, rk_out(c, (size_t)q * n + i, Ui[q] + du));
+        store_out(c, (size_t)q * D.n + es.i, rk_out(c, (size_t)q * D.n + es.i, Ui[q] + du));
       }
     }
   }
@@ -283,7 +285,6 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   // entries; half the FP64 operations of a loop in which every row does its own.
   // With dU^H = 0 the viscous part, which both rows have, is all there is; a row whose A is zero throughout is
   // marked instead of written: U^(1)_i = U^L_i whatever its factors, which are 1.
-  const int elem = valid ? div_nl(D, i) : 0;
   quiet = quiet && flat;
   if (flat && !quiet) {
     unsigned bit = 1;
@@ -296,14 +297,14 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   for (int e = flat ? r1 : r0; e < r1; e += kEll, bit <<= 1) {
     const int j = D.col[e];
     const bool visc = e < se && !(zeros & bit);
-    const int ej = div_nl(D, j);
-    if (ej != elem) {  // no mass term
+    const int sj = j / kEll, gj = div_nl(D, sj);  // slice and group of j
+    if (gj != es.g || ((j ^ i) & (kEll - 1)) != 0) {  // another element: no mass term
       if (!visc)
 #pragma unroll
         for (int q = 0; q < M; ++q) S.A[(size_t)q * D.nnz + e] = 0.0;
       continue;
     }
-    const int lj = j - ej * nl;
+    const int lj = sj - gj * nl;
     int after = lj - es.l;
     if (after < 0) after += nl;
     if (2 * after > nl || (2 * after == nl && lj < es.l)) continue;

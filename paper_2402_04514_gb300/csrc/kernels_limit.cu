@@ -23,9 +23,10 @@ __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last
   if (finished(c)) return;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const int i = row_node(D, lb * blockDim.x + threadIdx.x, sliced && !(last && c.Uhost));
-  if (i < 0) return;
-  const size_t n = D.n, nnz = D.nnz, nb = D.nb;
+  const Node nd = row_node(D, lb * blockDim.x + threadIdx.x, sliced && !(last && c.Uhost));
+  if (nd.i < 0) return;
+  const int i = nd.t;
+  const size_t n = D.ns, nnz = D.nnz, nb = D.nb;
   double acc[M];
 #pragma unroll
   for (int q = 0; q < M; ++q) acc[q] = 0.0;
@@ -50,7 +51,7 @@ __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last
   for (int q = 0; q < M; ++q) U1[q] = S.UL[q * n + i] + acc[q] * inv_mi;
   if (last) {
 #pragma unroll
-    for (int q = 0; q < M; ++q) store_out(c, q * n + i, rk_out(c, q * n + i, U1[q]));
+    for (int q = 0; q < M; ++q) store_out(c, (size_t)q * D.n + nd.i, rk_out(c, (size_t)q * D.n + nd.i, U1[q]));
     return;
   }
 #pragma unroll
@@ -110,7 +111,7 @@ __device__ __forceinline__ void lsfix_body(const Src& src, int pass) {
   const Dev& D = c.D;
   const Scratch& S = c.S;
   const unsigned count = S.lsq_n[pass];
-  const size_t n = D.n, nnz = D.nnz, nb = D.nb;
+  const size_t n = D.ns, nnz = D.nnz, nb = D.nb;
   const unsigned stride = (unsigned)blocks_per_inst * blockDim.x;
   const unsigned first = ((threadIdx.x >> 5) * (unsigned)blocks_per_inst + (unsigned)lb) * 32u + (threadIdx.x & 31u);
   for (unsigned k = first; k < count; k += stride) {
@@ -152,12 +153,13 @@ __device__ __forceinline__ void final_body(const Src& src, int sliced) {
   if (finished(c)) return;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const int i = row_node(D, lb * blockDim.x + threadIdx.x, sliced && !c.Uhost);
-  if (i < 0) return;
-  const size_t n = D.n, nnz = D.nnz, nb = D.nb;
+  const Node nd = row_node(D, lb * blockDim.x + threadIdx.x, sliced && !c.Uhost);
+  if (nd.i < 0) return;
+  const int i = nd.t;
+  const size_t n = D.ns, no = D.n, nnz = D.nnz, nb = D.nb;
   if (S.rem[i] != 1) {  // no remainder in the row: U^(2)_i = U^(1)_i
 #pragma unroll
-    for (int q = 0; q < M; ++q) store_out(c, q * n + i, rk_out(c, q * n + i, S.U1[q * n + i]));
+    for (int q = 0; q < M; ++q) store_out(c, q * no + nd.i, rk_out(c, q * no + nd.i, S.U1[q * n + i]));
     return;
   }
   double acc[M];
@@ -180,7 +182,7 @@ __device__ __forceinline__ void final_body(const Src& src, int sliced) {
   }
   const double inv_mi = D.inv_mi[i];
 #pragma unroll
-  for (int q = 0; q < M; ++q) store_out(c, q * n + i, rk_out(c, q * n + i, S.U1[q * n + i] + acc[q] * inv_mi));
+  for (int q = 0; q < M; ++q) store_out(c, q * no + nd.i, rk_out(c, q * no + nd.i, S.U1[q * n + i] + acc[q] * inv_mi));
 }
 
 template <int DIM, class Src>

@@ -28,12 +28,15 @@ __device__ __forceinline__ void prim_body(const Src& src) {
   if (done && !c.Ucopy) return;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const int i = lb * blockDim.x + threadIdx.x;
-  if (i == 0 && !done) {
+  const int slot = lb * blockDim.x + threadIdx.x;
+  if (slot == 0 && !done) {
     S.lsq_n[0] = 0u;
     S.lsq_n[1] = 0u;
   }
-  if (i >= D.n) return;
+  // by slots, so that the nine or more arrays written here are; over the host link the reads decide
+  const Node nd = row_node(D, slot, c.Ucopy == nullptr);
+  const int i = nd.i, t = nd.t;
+  if (i < 0) return;
   double Ui[DIM + 2];
   load_state<DIM>(c.U, D.n, i, Ui);
   if (c.Ucopy) {
@@ -46,6 +49,9 @@ __device__ __forceinline__ void prim_body(const Src& src) {
       return;
     }
   }
+  const size_t n = D.ns;
+#pragma unroll
+  for (int q = 0; q < DIM + 2; ++q) S.Us[q * n + t] = Ui[q];
   double irho = rcp64(Ui[0]);
   // products on the integer pipe (sf::mul, the same bits as the FP64 instruction) where no sum follows
   double m2 = sf::mul(Ui[1], Ui[1]);
@@ -55,7 +61,6 @@ __device__ __forceinline__ void prim_body(const Src& src) {
   if (!(Ui[0] > 0.0) || !(eps > 0.0)) atomicOr(S.flags, (unsigned)GDG_FLAG_INADMISSIBLE);
   double p = sf::mul(D.gm1, eps);
   double* P = S.prim;
-  size_t n = D.n;
   if constexpr (MX) {
     const PrimF f = prim_mx(D, Ui[0], p);
     float st = powf(to_f32(Ui[0]), -D.gamma_f) * to_f32(eps);
@@ -65,28 +70,28 @@ __device__ __forceinline__ void prim_body(const Src& src) {
       st64 = rho_neg_gamma(D, Ui[0], &ir) * eps;
       st = to_f32(st64);
     }
-    P[PR_IRHO * n + i] = irho;
-    P[PR_P * n + i] = p;
-    P[PR_IP * n + i] = to_f64(f.ip);
-    P[PR_A * n + i] = to_f64(f.a);
-    P[PR_PME * n + i] = to_f64(f.pme);
-    P[PR_F * n + i] = to_f64(powf(2.f * D.gm1h_f * st, D.inv_gp1_f));
-    P[PR_ST * n + i] = st64;
+    P[PR_IRHO * n + t] = irho;
+    P[PR_P * n + t] = p;
+    P[PR_IP * n + t] = to_f64(f.ip);
+    P[PR_A * n + t] = to_f64(f.a);
+    P[PR_PME * n + t] = to_f64(f.pme);
+    P[PR_F * n + t] = to_f64(powf(2.f * D.gm1h_f * st, D.inv_gp1_f));
+    P[PR_ST * n + t] = st64;
     return;
   }
   double ir;
   double st = sf::mul(rho_neg_gamma(D, Ui[0], &ir), eps);
-  P[PR_IRHO * n + i] = irho;
-  P[PR_P * n + i] = p;
-  P[PR_IP * n + i] = rcp64(p);
-  P[PR_A * n + i] = sqrt64(sf::mul(sf::mul(D.gamma, p), irho));
-  P[PR_PME * n + i] = D.ie_root > 0 ? rootinv(p, D.root_ie) : pow_hw(p, -D.e_exp);
+  P[PR_IRHO * n + t] = irho;
+  P[PR_P * n + t] = p;
+  P[PR_IP * n + t] = rcp64(p);
+  P[PR_A * n + t] = sqrt64(sf::mul(sf::mul(D.gamma, p), irho));
+  P[PR_PME * n + t] = D.ie_root > 0 ? rootinv(p, D.root_ie) : pow_hw(p, -D.e_exp);
   // f = (gm1 s~)^{1/(gamma+1)} = x^{q/(p+q)} = x (x^{-1/(p+q)})^p for gamma = p/q
   double x = sf::mul(D.gm1, st);
-  P[PR_F * n + i] = (D.gq > 0 && D.gp + D.gq <= 16 && sf::pos_normal(x))
+  P[PR_F * n + t] = (D.gq > 0 && D.gp + D.gq <= 16 && sf::pos_normal(x))
                         ? sf::uf_dbl(sf::uf_mul(sf::uf_of(x), sf::uf_pow(sf::uf_rootinv(x, D.root_gpq.c), D.gp)))
                         : pow_hw(x, D.inv_gp1);
-  P[PR_ST * n + i] = st;
+  P[PR_ST * n + t] = st;
 }
 
 template <int DIM, bool MX, class Src>
@@ -144,13 +149,13 @@ __device__ __forceinline__ void maxdt_body(const Src& src) {
   const Dev& D = c.D;
   const Scratch& S = c.S;
   const double* P = S.prim;
-  const size_t n = D.n, nnz = D.nnz;
+  const size_t n = D.ns, nnz = D.nnz;
   const unsigned slot = lb * blockDim.x + threadIdx.x, nbs = boundary_slots(D.nb);
   if (slot < nbs) {
     if (slot >= (unsigned)D.nb) return;
     const int i = D.bnode[slot];
     double Ui[M];
-    load_state<DIM>(c.U, D.n, i, Ui);
+    load_state<DIM>(S.Us, D.ns, i, Ui);
     S.bbar[slot] = boundary_viscosity<DIM, MX>(D, (int)slot, Ui, c.bdata, P[PR_IRHO * n + i], P[PR_P * n + i],
                                                P[PR_IP * n + i], P[PR_A * n + i], P[PR_PME * n + i]);
     return;
@@ -162,8 +167,8 @@ __device__ __forceinline__ void maxdt_body(const Src& src) {
 #pragma unroll
   for (int q = 0; q < DIM; ++q) {
     nv[q] = D.cn[q * nnz + e];
-    mi[q] = c.U[(1 + q) * n + i];
-    mj[q] = c.U[(1 + q) * n + j];
+    mi[q] = S.Us[(1 + q) * n + i];
+    mj[q] = S.Us[(1 + q) * n + j];
   }
   const double ir_i = P[PR_IRHO * n + i], ir_j = P[PR_IRHO * n + j];
   const double uL = sf::mul(dot<DIM>(mi, nv), ir_i), uR = sf::mul(dot<DIM>(mj, nv), ir_j);
@@ -192,11 +197,12 @@ __device__ __forceinline__ void tau_body(const Src& src, int sliced) {
   if (finished(c)) return;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const int i = row_node(D, lb * blockDim.x + threadIdx.x, sliced);
+  const Node nd = row_node(D, lb * blockDim.x + threadIdx.x, sliced);
+  const int i = nd.t;
   const double* dL = c.clk ? S.dL : S.barR;
   const double* dB = c.clk ? S.dB : S.bbar;
   double val = INFINITY;
-  if (i >= 0) {
+  if (nd.i >= 0) {
     double dsum = 0.0;
     const int e0 = D.rbeg[i], e1 = D.sten_end[i];
 #pragma unroll 4
@@ -238,11 +244,11 @@ __device__ __noinline__ void boundary_entry(const Ctx& c, int b) {
   constexpr int M = DIM + 2;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const size_t n = D.n, nb = D.nb;
+  const size_t n = D.ns, nb = D.nb;
   const int i = D.bnode[b];
   const double* P = S.prim;
   double Ui[M], nv[DIM], UB[M];
-  load_state<DIM>(c.U, D.n, i, Ui);
+  load_state<DIM>(S.Us, D.ns, i, Ui);
   const double irho_i = P[PR_IRHO * n + i], p_i = P[PR_P * n + i];
 #pragma unroll
   for (int k = 0; k < DIM; ++k) nv[k] = D.bn[(size_t)k * nb + b];
@@ -305,13 +311,13 @@ __device__ __forceinline__ void edge_body(const Src& src) {
   }
   const unsigned k = slot - nbs;
   if (k >= (unsigned)D.ne) return;
-  const size_t n = D.n, nnz = D.nnz;
+  const size_t n = D.ns, nnz = D.nnz;
   const int e = D.edge_e[k], i = D.edge_i[k];
   const int j = D.col[e], t = D.tr[e];
   const double* P = S.prim;
   double Ui[M], Uj[M], nv[DIM];
-  load_state<DIM>(c.U, D.n, i, Ui);
-  load_state<DIM>(c.U, D.n, j, Uj);
+  load_state<DIM>(S.Us, D.ns, i, Ui);
+  load_state<DIM>(S.Us, D.ns, j, Uj);
   const double cnm = D.cnorm[e];
   // products on the integer pipe (sf::mul, the same bits as the FP64 instruction) where no sum follows
 #pragma unroll
@@ -412,14 +418,15 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
   if (finished(c)) return;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const double* U = c.U;
-  const int i = row_node(D, lb * blockDim.x + threadIdx.x, sliced && !(write_out && c.Uhost));
-  if (i < 0) return;
+  const double* U = S.Us;
+  const Node nd = row_node(D, lb * blockDim.x + threadIdx.x, sliced && !(write_out && c.Uhost));
+  if (nd.i < 0) return;
+  const int i = nd.t;
   const double tau = stage_tau(c);
-  size_t n = D.n;
+  size_t n = D.ns;
   const double* P = S.prim;
   double Ui[M];
-  load_state<DIM>(U, D.n, i, Ui);
+  load_state<DIM>(U, D.ns, i, Ui);
   const double irho_i = P[PR_IRHO * n + i], ip_i = P[PR_IP * n + i], f_i = P[PR_F * n + i],
                st_i = P[PR_ST * n + i];
   using Acc = std::conditional_t<MX, float, double>;  // arithmetic of the indicator's sums
@@ -444,7 +451,7 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
     const double d = S.dL[e];
     dsum += d;
     double Uj[M];
-    load_state<DIM>(U, D.n, j, Uj);
+    load_state<DIM>(U, D.ns, j, Uj);
     bool same = true;
 #pragma unroll
     for (int q = 0; q < M; ++q) same = same && same_bits(Ui[q], Uj[q]);
@@ -506,7 +513,7 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
   }
   if (write_out) {
 #pragma unroll
-    for (int q = 0; q < M; ++q) store_out(c, (size_t)q * n + i, rk_out(c, (size_t)q * n + i, UL[q]));
+    for (int q = 0; q < M; ++q) store_out(c, (size_t)q * D.n + nd.i, rk_out(c, (size_t)q * D.n + nd.i, UL[q]));
     return;
   }
 #pragma unroll
