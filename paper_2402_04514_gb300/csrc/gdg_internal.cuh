@@ -419,6 +419,11 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, int block, cudaS
   return cudaGetLastError();
 }
 
+// Whether a launch has too few threads to fill the SMs (24 warps each) even at a high register count: the row and
+// element sweeps then take the instantiation without their tight register cap, whose spills cost a short chain of
+// work more than the occupancy it does not need (Q2 33 x 47: 440 us against 455 per step).
+inline bool few_threads(long long blocks, int threads) { return blocks * threads <= 152LL * 768; }
+
 // Kernel launchers of each file, dim in 1..3: one instance (context by value) or a batch (Many; blocks =
 // the batch's total for that kernel).  arg: write_out for KN_LOW (the stage ends after U^L), last for
 // KN_LIMIT2 (one limiter pass only), the pass (0 or 1) for KN_LSFIX.  threads: the block size of a

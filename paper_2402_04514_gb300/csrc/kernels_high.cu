@@ -376,17 +376,22 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   }
 }
 
-// The element sweep of each path as its own kernel with its own register budget.  Both run fastest at 72
-// registers (three 288-thread blocks per SM, a few spills): with the per-entry streams contiguous, the
-// resident warps matter more than the spills (the mixed path took 3.97 ms per launch at 96 registers,
-// 3.37 ms at 72, at 1024^2 Q2; with the integer-pipe products the FP64 path 4.36 ms at 64, 4.15 at 72).
+// The element sweep of each path as its own kernel with its own register budget.  Its loads, FP64 chains and 64-bit
+// integer chains leave the issue slots half empty at 27 warps per SM, so a few spills are worth a fourth 288-thread
+// block: in us per launch at 72, 56 and 48 registers 1,384, 1,231 and 1,185 (Q2 1024^2), 133, 99 and 104 (Q3 96^2), 240, 238
+// and 254 (Q1 512^2), 380, 372 and 357 (Q1 48 x 40 x 44); the mixed path 300, 261 and 242 (Q2 384^2).
 template <int DIM, class Src>
-__global__ void __maxnreg__(72) k_high(Src src, int eb) {
+__global__ void __maxnreg__(56) k_high(Src src, int eb) {
   chain_begin();
   high_sweep<DIM, false, Src>(src, eb);
 }
 template <int DIM, class Src>
-__global__ void __maxnreg__(72) k_high_mixed(Src src, int eb) {
+__global__ void __maxnreg__(72) k_high_few(Src src, int eb) {
+  chain_begin();
+  high_sweep<DIM, false, Src>(src, eb);
+}
+template <int DIM, class Src>
+__global__ void __maxnreg__(48) k_high_mixed(Src src, int eb) {
   chain_begin();
   high_sweep<DIM, true, Src>(src, eb);
 }
@@ -399,10 +404,13 @@ cudaError_t high_launch(const Src& src, long long blocks, int n_loc, int eb, cud
   if (eb < 1 || eb > kEll || (eb & (eb - 1)) || n_loc < 1 || n_loc > kMaxLocal || eb * n_loc > kMaxBlock)
     return cudaErrorInvalidValue;
   const int threads = high_threads(n_loc, eb);
-  if constexpr (MX)
+  if constexpr (MX) {
     return launch_chained(k_high_mixed<DIM, Src>, (unsigned)blocks, threads, s, src, eb);
-  else
+  } else {
+    if constexpr (std::is_same_v<Src, One>)
+      if (few_threads(blocks, threads)) return launch_chained(k_high_few<DIM, Src>, (unsigned)blocks, threads, s, src, eb);
     return launch_chained(k_high<DIM, Src>, (unsigned)blocks, threads, s, src, eb);
+  }
 }
 
 template <class Src>

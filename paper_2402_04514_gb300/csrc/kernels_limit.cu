@@ -1,5 +1,7 @@
 // Sweeps C and D: symmetrisation of the limiter coefficients, the limited updates of Sec. 5.3,
 // eq. (LimitedScheme), and the second limiter pass of Sec. 6.1.  One thread per row.
+#include <type_traits>
+
 #include "gdg_internal.cuh"
 
 namespace gdg {
@@ -11,9 +13,9 @@ constexpr int kLimThreads = kRowMaxThreads;  // launch bound; the schedule launc
 // Sweep C: l_ij = min(l_ij^(i), l_ji^(j)) (Lemma ConsInvariants needs l_ij = l_ji);
 // U^(1)_i = U^L_i + (sum_j l_ij A_ij + sum_k l_i^k A_i^k) / m_i; then the second pass limits the
 // remainder (1 - l) A from U^(1) against the same bounds.  With one pass it writes U_out from U^(1).
-// Capped at 72 registers (seven 128-thread blocks per SM; a few bytes of spills in the search): the row
-// sums, which every row runs, need far fewer, and the searches of the rare rows with a remainder would
-// otherwise set the kernel's occupancy.
+// Capped at 48 registers (five 256-thread blocks per SM): the row sums, which every row runs, need fewer, and wait for
+// memory; the searches of the rare rows with a remainder would otherwise set the kernel's occupancy.  In us per
+// launch at 72, 48 and 40 registers: 422, 341 and 327 (Q2 1024^2), 72, 62 and 62 (Q1 512^2), 36, 35 and 38 (Q3 96^2).
 template <int DIM, class Src>
 __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last) {
   constexpr int M = DIM + 2;
@@ -91,7 +93,12 @@ __device__ __forceinline__ void limit2_body(const Src& src, int sliced, int last
 }
 
 template <int DIM, class Src>
-__global__ void __maxnreg__(72) k_limit2(Src src, int sliced, int last) {
+__global__ void __maxnreg__(48) k_limit2(Src src, int sliced, int last) {
+  chain_begin();
+  limit2_body<DIM, Src>(src, sliced, last);
+}
+template <int DIM, class Src>
+__global__ void __maxnreg__(72) k_limit2_few(Src src, int sliced, int last) {
   chain_begin();
   limit2_body<DIM, Src>(src, sliced, last);
 }
@@ -253,7 +260,10 @@ cudaError_t limit_launch(int kern, const Src& src, long long blocks, int threads
   if (threads < 32 || threads > kLimThreads || threads % 32) return cudaErrorInvalidValue;
   const unsigned g = (unsigned)blocks;
   switch (kern) {
-    case KN_LIMIT2: return launch_chained(k_limit2<DIM, Src>, g, threads, s, src, sliced, arg);
+    case KN_LIMIT2:
+      if constexpr (std::is_same_v<Src, One>)
+        if (few_threads(blocks, threads)) return launch_chained(k_limit2_few<DIM, Src>, g, threads, s, src, sliced, arg);
+      return launch_chained(k_limit2<DIM, Src>, g, threads, s, src, sliced, arg);
     case KN_FINAL: return launch_chained(k_final<DIM, Src>, g, threads, s, src, sliced);
     case KN_AXPY: return launch_chained(k_axpy<DIM, Src>, g, threads, s, src);
     case KN_LSFIX: return launch_chained(k_lsfix<DIM, Src>, g, kLsfixThreads, s, src, arg);

@@ -578,8 +578,16 @@ __device__ __forceinline__ void low_body(const Src& src, int sliced, int write_o
   }
 }
 
+// Four 256-thread blocks per SM (three in 3D): the row sums wait for loads and for the FP64 pipe.  In us per launch at
+// 78 to 106 registers, at 64 (80) and at 48 (64): 845, 728 and 745 (Q2 1024^2), 181, 175 and 178 (Q1 512^2), 218, 206 and
+// 208 (Q1 48 x 40 x 44); mixed 209, 154 and 166 (Q2 384^2).
 template <int DIM, bool MX, class Src>
-__global__ void __launch_bounds__(kThreads) k_low(Src src, int sliced, int write_out) {
+__global__ void __maxnreg__(DIM == 3 ? 80 : 64) k_low(Src src, int sliced, int write_out) {
+  chain_begin();
+  low_body<DIM, MX, Src>(src, sliced, write_out);
+}
+template <int DIM, bool MX, class Src>
+__global__ void __launch_bounds__(kThreads) k_low_few(Src src, int sliced, int write_out) {
   chain_begin();
   low_body<DIM, MX, Src>(src, sliced, write_out);
 }
@@ -594,7 +602,10 @@ cudaError_t low_launch(int kern, const Src& src, long long blocks, int threads, 
     case KN_MAXDT: return launch_chained(k_maxdt<DIM, MX, Src>, g, threads, s, src);
     case KN_TAU: return launch_chained(k_tau<DIM, MX, Src>, g, threads, s, src, sliced);
     case KN_EDGE: return launch_chained(k_edge<DIM, MX, Src>, g, threads, s, src);
-    case KN_LOW: return launch_chained(k_low<DIM, MX, Src>, g, threads, s, src, sliced, arg);
+    case KN_LOW:
+      if constexpr (std::is_same_v<Src, One>)
+        if (few_threads(blocks, threads)) return launch_chained(k_low_few<DIM, MX, Src>, g, threads, s, src, sliced, arg);
+      return launch_chained(k_low<DIM, MX, Src>, g, threads, s, src, sliced, arg);
     default: return cudaErrorInvalidValue;
   }
 }
