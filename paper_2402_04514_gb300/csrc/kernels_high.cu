@@ -48,8 +48,8 @@ __device__ __forceinline__ ElemSlot element_slot(const Dev& D, int lb, int eb) {
 //     its stencil neighbours and node i's own boundary bar states;
 //  4. A_ij = tau (d^H_ij - d^L_ij)(U_j - U_i) - m_ij (dU^H_j - dU^H_i) and
 //     A_i^{d,k} = tau (d^{d,H} - d^{d,L})(U^{d,k} - U_i) (Sec. 5.3, eq. (HighLowOrderIdentity)), and the
-//     pass-1 line search of Sec. 5.4, eq. (ConvexScheme), from U^L with P = A / (kappa_i m_i); the rare
-//     searches that need the bracketed iteration are queued for k_lsfix.
+//     pass-1 line search of Sec. 5.4, eq. (ConvexScheme), from U^L with P = A / (kappa_i m_i); the
+//     searches that FP32 does not settle are queued for k_lsfix.
 // With order HIGH the kernel stops after 2 and writes U_out = alpha U_base + (1 - alpha)(U + dU^H).
 // The mixed path (MX) runs steps 1, 2 and the A_ij of step 4 in FP32 (the differences U_j - U_i in FP64
 // first); the bounds and the line search stay FP64.
