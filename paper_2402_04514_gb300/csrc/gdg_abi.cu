@@ -155,7 +155,10 @@ int64_t node_slot(int64_t i, int nl) {
 template <class T>
 std::vector<T> by_slot(const std::vector<T>& a, int nl, int64_t ns) {
   std::vector<T> r((size_t)ns, T(0));
-  for (int64_t i = 0; i < (int64_t)a.size(); ++i) r[(size_t)node_slot(i, nl)] = a[(size_t)i];
+  parallel_for((int64_t)a.size() / nl, [&](int64_t b, int64_t e) {
+    for (int64_t E = b; E < e; ++E)
+      for (int l = 0; l < nl; ++l) r[(size_t)(node_slot(E * nl, nl) + l * gdg::kEll)] = a[(size_t)(E * nl + l)];
+  });
   return r;
 }
 
@@ -488,13 +491,18 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
         h->epos[q] = (int)(p0 + gdg::kEll * (int64_t)(q - h->row_ptr[i]));
     }
   });
+  std::vector<int> slot(n);  // of every node
+  parallel_for(nel, [&](int64_t b, int64_t e) {
+    for (int64_t E = b; E < e; ++E)
+      for (int l = 0; l < nl; ++l) slot[E * nl + l] = (int)(node_slot(E * nl, nl) + l * gdg::kEll);
+  });
   // the per-entry arrays in ELL order; padding slots stay zero and no kernel reads them
   std::vector<int> col_e((size_t)NE, 0), tr_e((size_t)NE, 0);
   std::vector<double> cnorm_e((size_t)NE, 0.0), cn_e((size_t)dim * NE, 0.0), mij_e((size_t)NE, 0.0);
   parallel_for(nnz, [&](int64_t b, int64_t e) {
     for (int64_t q = b; q < e; ++q) {
       const int64_t pq = h->epos[q];
-      col_e[pq] = (int)node_slot(h->col[q], nl);
+      col_e[pq] = slot[h->col[q]];
       tr_e[pq] = h->epos[h->tr[q]];
       cnorm_e[pq] = cnorm[q];
       mij_e[pq] = mij[q];
@@ -529,7 +537,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   std::vector<int> edge_e(edges.size()), edge_i(edges.size());
   for (size_t k = 0; k < edges.size(); ++k) {
     edge_e[k] = edges[k].first;
-    edge_i[k] = (int)node_slot(edges[k].second, nl);
+    edge_i[k] = slot[edges[k].second];
   }
   const int64_t ne = (int64_t)edge_e.size();
   // the boundary entries in the order of their nodes' slots, the caller's order within a node
