@@ -49,14 +49,19 @@ SF_FN float flt(uint32_t u) {
 #endif
 }
 
-// The special-function unit's approximations (relative error below 2^-22 for the arguments they get here).
+// The special-function unit's approximations (relative error below 2^-22 for the arguments they get here).  On the host
+// rounded double values stand for them, passed through SF_HOST_APPROX, by which a check can move them within the
+// instructions' documented errors.
+#ifndef SF_HOST_APPROX
+#define SF_HOST_APPROX(y) (y)
+#endif
 SF_FN float mufu_rcp(float x) {
 #if defined(__CUDA_ARCH__)
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 #else
-  return 1.0f / x;
+  return (float)SF_HOST_APPROX(1.0 / x);
 #endif
 }
 SF_FN float mufu_rsqrt(float x) {
@@ -65,7 +70,7 @@ SF_FN float mufu_rsqrt(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 #else
-  return 1.0f / sqrtf(x);
+  return (float)SF_HOST_APPROX(1.0 / sqrt((double)x));
 #endif
 }
 SF_FN float mufu_lg2(float x) {
@@ -74,7 +79,7 @@ SF_FN float mufu_lg2(float x) {
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 #else
-  return log2f(x);
+  return (float)SF_HOST_APPROX(log2((double)x));
 #endif
 }
 SF_FN float mufu_ex2(float x) {
@@ -83,7 +88,7 @@ SF_FN float mufu_ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 #else
-  return exp2f(x);
+  return (float)SF_HOST_APPROX(exp2((double)x));
 #endif
 }
 
@@ -133,13 +138,20 @@ SF_FN uf uf_pow(uf x, int k) {
   return r;
 }
 
+// The 24-bit significand of an approximation y of a number in [1/2, 1], in units of 2^-24.  y itself may lie an ulp or two below
+// 1/2 (the reciprocal of a number just below 2, the inverse square root of one just below 4), where its exponent
+// would give a negative shift: 1/2 is then the better approximation.
+SF_FN uint32_t sig_half(float y) {
+  const uint32_t u = fbits(y), b = u < 0x3f000000u ? 0x3f000000u : u;
+  return ((b & 0x7fffffu) | 0x800000u) << ((b >> 23) - 126u);
+}
+
 // 1 / m for the significand m of x in [1, 2), in units of 2^-63: at most 2^63, which m = 1 gives.  With Y the
 // 24-bit approximation and e = 1 - m Y (below 2^-21), 1 / m = Y (1 + e + e^2 + ...): the residual
 // -M Y modulo 2^64 (M Y is near 2^76, a multiple of 2^64), then Y e and Y e^2; Y e^3 is below 2^-63.
 SF_FN uint64_t rcp_sig(double x) {
   const uint32_t mh = (hiw(x) & 0xfffffu) | 0x100000u, ml = low(x);
-  const uint32_t b = fbits(mufu_rcp(sigf(x)));  // in [1/2, 1]
-  const uint32_t Y = ((b & 0x7fffffu) | 0x800000u) << ((b >> 23) - 126u);
+  const uint32_t Y = sig_half(mufu_rcp(sigf(x)));
   const uint64_t MY = wide(ml, Y) + ((uint64_t)(mh * Y) << 32);
   const int64_t r = -(int64_t)MY;  // e in units of 2^-76
   const int32_t rh = (int32_t)(r >> 32);
@@ -170,8 +182,7 @@ SF_FN uf uf_rcp(double x) {  // positive normal x
 SF_FN double sqrt_pos(double x) {
   const int ex = expo(x), odd = (ex & 1) ^ 1;  // 1023 is odd: an even field is an odd power of two
   const uint64_t X = sig53(x) << odd;          // units of 2^-52, below 2^54
-  const uint32_t b = fbits(mufu_rsqrt(flt(fbits(sigf(x)) + ((uint32_t)odd << 23))));  // in [1/2, 1]
-  const uint32_t Y = ((b & 0x7fffffu) | 0x800000u) << ((b >> 23) - 126u);          // units of 2^-24
+  const uint32_t Y = sig_half(mufu_rsqrt(flt(fbits(sigf(x)) + ((uint32_t)odd << 23))));
   const uint32_t xh = (uint32_t)(X >> 32), xl = (uint32_t)X;
   // s = X Y in units of 2^-60: (X Y) >> 16, X Y below 2^78
   const uint64_t p0 = wide(xl, Y), p1 = wide(xh, Y) + (p0 >> 32);
