@@ -102,7 +102,7 @@ struct Arena {
   X(rbeg, int, n) X(rend, int, n) X(sten, int, n) X(col, int, nnz) X(tr, int, nnz) X(cnorm, double, nnz) X(cn, double, dim * nnz)   \
   X(mij, double, nnz) X(mu, double, nnz) X(mi, double, n) X(imi, double, n) X(ikm, double, n)             \
   X(rm, double, n) X(rp, double, n) X(muB, double, n) X(bptr, int, n + 1) X(bnorm, double, nb)           \
-  X(bn, double, dim * nb) X(btype, int, nb) X(borig, int, nb) X(bnode, int, nb) X(minv, double, nel * nl * nl) X(wexp, int, n)             \
+  X(bn, double, dim * nb) X(btype, int, nb) X(borig, int, nb) X(bnode, int, nb) X(minv, double, nel * nl * nl)             \
   X(ee, int, ne) X(ei, int, ne) X(G, double, m * nnz) X(psi, double, nnz) X(barR, double, nnz) X(barS, double, nnz)          \
   X(prim, double, gdg::NPRIM * n) X(dL, double, nnz) X(dB, double, nb) X(bbar, double, 2 * nb)            \
   X(UB, double, m * nb) X(gB, double, m * nb) X(gI, double, m * nb)                                       \
@@ -511,20 +511,13 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   });
   // M_K^{-1} grouped like the entries: (K, a, b) at ((K / kEll * nl + a) * nl + b) * kEll + K % kEll
   const int64_t nel_pad = padded_elements(nel);
-  // every row in fixed point below its own power of two (fixfp64.cuh, fix56), whose exponent field goes to wexp
-  std::vector<sf::fixp> minv_g((size_t)nel_pad * nl * nl, sf::fixp{0, 0});
-  std::vector<int> wexp(n, 0);
+  std::vector<double> minv_g((size_t)nel_pad * nl * nl, 0.0);
   parallel_for(nel, [&](int64_t b, int64_t e) {
     for (int64_t K = b; K < e; ++K)
-      for (int a = 0; a < nl; ++a) {
-        const double* row = MKinv.data() + ((size_t)K * nl + a) * nl;
-        int E = 0;
-        for (int c = 0; c < nl; ++c) E = std::max(E, sf::expo(row[c]));
-        wexp[K * nl + a] = E;
+      for (int a = 0; a < nl; ++a)
         for (int c = 0; c < nl; ++c)
           minv_g[(((size_t)(K / gdg::kEll) * nl + a) * nl + c) * gdg::kEll + K % gdg::kEll] =
-              sf::fix_parts(sf::fix56(row[c], E));
-      }
+              MKinv[((size_t)K * nl + a) * nl + c];
   });
   // canonical stencil edges (i < j, c_ij != 0) in ELL order: consecutive threads of the edge sweep take
   // the same entry of the rows of consecutive elements, so their per-entry writes are contiguous
@@ -600,8 +593,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
       (ce = up(o_btype, btype.data(), sizeof(int) * nb)) != cudaSuccess ||
       (ce = up(o_borig, border.data(), sizeof(int) * nb)) != cudaSuccess ||
       (ce = up(o_bnode, bnode.data(), sizeof(int) * nb)) != cudaSuccess ||
-      (ce = up(o_minv, minv_g.data(), sizeof(sf::fixp) * minv_g.size())) != cudaSuccess ||
-      (ce = up(o_wexp, by_slot(wexp, nl, ns).data(), sizeof(int) * ns)) != cudaSuccess ||
+      (ce = up(o_minv, minv_g.data(), sizeof(double) * minv_g.size())) != cudaSuccess ||
       (ce = up(o_ee, edge_e.data(), sizeof(int) * ne)) != cudaSuccess ||
       (ce = up(o_ei, edge_i.data(), sizeof(int) * ne)) != cudaSuccess ||
       (ce = cudaMemset(ptr(o_flags), 0, 16)) != cudaSuccess)
@@ -636,8 +628,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   D.btype = (const int*)ptr(o_btype);
   D.borig = (const int*)ptr(o_borig);
   D.bnode = (const int*)ptr(o_bnode);
-  D.MKinv = (const int2*)ptr(o_minv);
-  D.wexp = (const int*)ptr(o_wexp);
+  D.MKinv = (const double*)ptr(o_minv);
   D.ne = (int)ne;
   D.edge_e = (const int*)ptr(o_ee);
   D.edge_i = (const int*)ptr(o_ei);

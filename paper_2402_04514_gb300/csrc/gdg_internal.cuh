@@ -63,8 +63,7 @@ struct Dev {
   const int* btype;     // [nb]
   const int* borig;     // [nb] index of the entry in the caller's order (for Dirichlet data)
   const int* bnode;     // [nb] node of the entry
-  const int2* MKinv;    // [n / n_loc][n_loc][n_loc] rows of M_K^{-1} in fixed point (sf::fixp)
-  const int* wexp;      // [ns] exponent field of the largest entry of each row
+  const double* MKinv;  // [n / n_loc][n_loc][n_loc] M_K^{-1}, grouped like the entries
   // canonical stencil edges: entries (i, j) with c_ij != 0 and i < j, in entry order
   int ne;
   const int* edge_e;    // [ne] entry index of (i, j)

@@ -59,7 +59,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   constexpr int kShared = kMaxBlock + kEll;        // room for one pad slot per element
   using R = std::conditional_t<MX, float, double>;  // arithmetic of steps 1, 2 and the A_ij of step 4
   __shared__ R sR[M][kShared];
-  __shared__ int sE[M][kEll];  // exponent field of the largest right-hand side of each element, 0 where all are zero
+  __shared__ int sE[kEll];  // 1 where some right-hand side of the element is not zero
   __shared__ R sdU[M][kShared];
   __shared__ Ctx sctx;
   int lb;
@@ -78,7 +78,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   const int sh = t0 + es.l;
   const size_t n = D.ns;
   const double tau = stage_tau(c);
-  for (int k = threadIdx.x; k < M * kEll; k += blockDim.x) (&sE[0][0])[k] = 0;
+  for (int k = threadIdx.x; k < kEll; k += blockDim.x) sE[k] = 0;
   __syncthreads();
   const R tau_r = MX ? R(to_f32(tau)) : R(tau);
   double Ui[M];
@@ -181,17 +181,16 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
         S.AB[(size_t)q * D.nb + b] = tau * dd * (UB[q] - Ui[q]);
       }
     }
+    bool zero = true;
 #pragma unroll
     for (int q = 0; q < M; ++q) {
-      int ex;
-      if constexpr (MX) {
-        sR[q][sh] = rhs[q];
-        ex = (int)(__float_as_uint(rhs[q]) & 0x7fffffffu);
-      } else {
-        ex = sf::expo(rhs[q]);
-      }
-      if (ex > 0) atomicMax(&sE[q][es.el], ex);
+      sR[q][sh] = rhs[q];
+      if constexpr (MX)
+        zero = zero && (__float_as_uint(rhs[q]) << 1) == 0u;
+      else
+        zero = zero && is_zero_bits(rhs[q]);
     }
+    if (!zero) sE[es.el] = 1;
     if (lim) {  // relaxed local bounds, read back after the solve
       double rmin = 0.0, rmax = INFINITY, smin = 0.0;
       if (D.bounds_mode == 0) {
@@ -206,60 +205,36 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
   }
   __syncthreads();
   // all right-hand sides of the element zero: so are dU^H and the mass terms of A
-  bool flat = true;
-#pragma unroll
-  for (int q = 0; q < M; ++q) flat = flat && sE[q][es.el] == 0;
-  if constexpr (!MX) {  // the right-hand sides in fixed point, in the place of the doubles
-    if (valid && !flat) {
-#pragma unroll
-      for (int q = 0; q < M; ++q) {
-        const sf::fixp f = sf::fix_parts(sf::fix56(rhs[q], sE[q][es.el]));
-        sR[q][sh] = __hiloint2double(f.hi, f.lo);
-      }
-    }
-    __syncthreads();
-  }
+  const bool flat = sE[es.el] == 0;
   if (valid) {
     const int nl = D.n_loc;
     // row il of the element's M_K^{-1}, stored grouped like the entries: (E, a, b) at
     // ((E / kEll * n_loc + a) * n_loc + b) * kEll + E % kEll
-    const int2* Minv = D.MKinv + ((size_t)es.g * nl + es.l) * nl * kEll + (i & (kEll - 1));
-    const int we = D.wexp[i];
+    const double* Minv = D.MKinv + ((size_t)es.g * nl + es.l) * nl * kEll + (i & (kEll - 1));
     if (flat) {
 #pragma unroll
       for (int q = 0; q < M; ++q) dUi[q] = R(0);
-    } else if constexpr (MX) {
+    } else {
+      // FP64 multiply-adds, 36 of the kernel's 130 operations per node (Q2 quads).  In fixed point on the integer pipe
+      // they are either less exact or no faster (fixdot.cuh).
       R acc[M];
 #pragma unroll
       for (int q = 0; q < M; ++q) acc[q] = R(0);
       for (int l = 0; l < nl; ++l) {
-        const int2 wf = __ldg(Minv + (size_t)l * kEll);
-        // in units of 2^(we - 1022), truncated like to_f32
-        const float w = __ll2float_rz(((long long)wf.x << 28) + wf.y) * 0x1p-56f;
+        R w;
+        if constexpr (MX)
+          w = to_f32(__ldg(Minv + (size_t)l * kEll));
+        else
+          w = __ldg(Minv + (size_t)l * kEll);
 #pragma unroll
         for (int q = 0; q < M; ++q) acc[q] += w * sR[q][t0 + l];
       }
 #pragma unroll
-      for (int q = 0; q < M; ++q) dUi[q] = -tau_r * to_f32(sf::mul_pow2(to_f64(acc[q]), we - 1022));
-    } else {
-      // fixed point (fixfp64.cuh): as FP64 multiply-adds this loop held the FP64 pipe, which bounds the kernel, for
-      // 36 of its 162 operations per node (Q2 quads); with the pairs of A below, k_high went from 3.68 to 3.20 ms
-      // per launch at Q2 1024^2 and from 555 to 488 us at Q1 48 x 40 x 44
-      sf::fixs s[M];
-#pragma unroll
-      for (int q = 0; q < M; ++q) s[q] = sf::fixs{0, 0, 0};
-      for (int l = 0; l < nl; ++l) {
-        const int2 wf = __ldg(Minv + (size_t)l * kEll);
-#pragma unroll
-        for (int q = 0; q < M; ++q) {
-          const double r = sR[q][t0 + l];
-          sf::fix_mad(sf::fixp{wf.x, wf.y}, sf::fixp{__double2hiint(r), __double2loint(r)}, s[q]);
-        }
-      }
-#pragma unroll
       for (int q = 0; q < M; ++q) {
-        const int re = sE[q][es.el];
-        dUi[q] = re < 0x7ff ? sf::mul(sf::neg(tau), sf::fix_dbl(s[q], we, re)) : __longlong_as_double(0x7ff8000000000000LL);
+        if constexpr (MX)
+          dUi[q] = -tau_r * acc[q];
+        else
+          dUi[q] = -tau * acc[q];
       }
     }
 #pragma unroll
@@ -272,7 +247,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
           du = to_f64(dUi[q]);
         else
           du = dUi[q];
-        store_out(c, (size_t)q * D.n + es.i, rk_out(c, (size_t)q * D.n + es.i, Ui[q] + du));
+        store_out(c, (size_t)q * D.n + es.i, rk_out(c, (size_t)q * D.n + es.i, U[(size_t)q * n + i] + du));
       }
     }
   }
