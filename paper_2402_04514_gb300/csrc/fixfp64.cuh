@@ -176,6 +176,26 @@ SF_FN uf uf_rcp(double x) {  // positive normal x
   return uf{T << (1 - one), 1022 - expo(x) + one};
 }
 
+// a / b for normal a and b with a quotient well inside the normal range (quot_ok), correctly rounded: a 53-bit quotient from
+// the reciprocal, at most one off, and the exact remainder, whose size says whether it is and how to round (a quotient
+// of two 53-bit numbers is never half way between two others).
+SF_FN bool quot_ok(double a, double b) {
+  const int ea = expo(a), eb = expo(b);
+  return (unsigned)(ea - 1) < 2046u && (unsigned)(eb - 1) < 2046u && (unsigned)(ea - eb + 1000) < 2000u;
+}
+SF_FN double quot(double a, double b) {
+  const uint64_t A = sig53(a), B = sig53(b);
+  const int below = A < B;                                              // the quotient of the significands is below 1
+  uint64_t q = mulhi64(A << 11, rcp_sig(b)) >> (10 - below);            // in units of 2^-52, below 1 of 2^-53
+  int64_t r = (int64_t)((A << (52 + below)) - q * B);                   // modulo 2^64; between -B and 2 B
+  const int less = r < 0, more = r >= (int64_t)B;
+  q += (uint64_t)more - (uint64_t)less;
+  r += less ? (int64_t)B : more ? -(int64_t)B : 0;
+  q += 2 * r > (int64_t)B;  // 2^53 after a carry: the addition below moves it on
+  const uint64_t e = (uint64_t)(uint32_t)(expo(a) - expo(b) + 1022 - below);
+  return dbl(((e << 52) + q) | ((uint64_t)((hiw(a) ^ hiw(b)) & 0x80000000u) << 32));
+}
+
 // sqrt(x) for a positive normal x.  X in [1, 4) is x with an even power of two taken out, Y the 24-bit
 // approximation of X^{-1/2}, s = X Y and e = 1 - s Y (below 2^-20): sqrt(X) = s (1 - e)^{-1/2} =
 // s (1 + e/2 + 3/8 e^2 + ...), the next term below 2^-61.

@@ -541,6 +541,11 @@ __device__ __forceinline__ double rcp64(double x) {
   if (__builtin_expect(!sf::rcp_ok(x), 0)) return rcp_hw(x);
   return sf::rcp(x);
 }
+static __device__ __noinline__ __attribute__((const)) double quot_hw(double x, double y) { return x / y; }
+__device__ __forceinline__ double quot64(double x, double y) {  // x / y, the same bits
+  if (__builtin_expect(!sf::quot_ok(x, y), 0)) return quot_hw(x, y);
+  return sf::quot(x, y);
+}
 __device__ __forceinline__ double sqrt64(double x) {
   if (__builtin_expect(!sf::pos_normal(x), 0)) return sqrt_hw(x);
   return sf::sqrt_pos(x);
@@ -982,12 +987,13 @@ __device__ __forceinline__ bool ls_certified(const Dev& D, const LsRow<DIM>& c, 
   return t > 1e-4f * scale + 1e-6f * fabsf(c.psi0f);
 }
 
-// The largest factor that the density bounds allow, in closed form, Pr = w A_rho.
+// The largest factor that the density bounds allow, in closed form, Pr = w A_rho.  One correctly rounded quotient: a product
+// with a rounded reciprocal is up to an ulp further off, by which rho(U0) + l Pr may pass its bound.
 __device__ __forceinline__ double ls_density(double rho, double Pr, double rmin, double rmax) {
   const double r1 = rho + Pr;
+  const bool above = r1 > rmax;
   double l = 1.0;
-  if (r1 < rmin) l = sf::mul(rmin - rho, rcp64(Pr));
-  if (r1 > rmax) l = sf::mul(rmax - rho, rcp64(Pr));
+  if (above || r1 < rmin) l = quot64((above ? rmax : rmin) - rho, Pr);
   if (__double_as_longlong(l) <= 0) l = 0.0;  // comparisons with 0 and 1 on the integer pipe
   return pmin(l, 1.0);
 }
