@@ -67,7 +67,10 @@ enum { GDG_PRECISION_FP64 = 0, GDG_PRECISION_MIXED = 1 };
 /* Method parameters.  gdg_default_params fills the paper's values: c_k = 1 and p_k = 1/2 (k even),
  * 0 (k odd) of Sec. 5.1; c_ev = 1, 0.5, 0.25 for k = 1, 2, >= 3 (Sec. 5.2); c_r = 4, p_r = 1.5
  * (Sec. 5.4, eq. (ViscMinConst2)); two limiter passes (Sec. 6.1); line-search bracket tolerance
- * 1e-14 with at most 50 iterations. */
+ * 1e-14 with at most 50 iterations.  ls_tol, ls_maxit: a line search ends at a feasible point within ls_tol of its root, or
+ * within the rounding of the entropy constraint psi (2^-52 E / |psi'|) where that is wider.  With ls_maxit >= 8 it starts with
+ * Newton steps, eight at most, and usually ends there; ls_maxit bounds the bracketed iteration (three
+ * evaluations each, or fewer) which follows where they do not settle, and which is all there is with ls_maxit < 8. */
 typedef struct {
   int32_t order;          /* GDG_ORDER_LOW: eq. (cijdijscheme) only; GDG_ORDER_HIGH: eq. (HighScheme)
                              without limiting; GDG_ORDER_LIMITED: eq. (LimitedScheme) */
@@ -214,8 +217,8 @@ int gdg_status(gdg_handle* h, int32_t* flags, int32_t clear, void* stream);
  * "l2" [nnz] (written only where min(l1_ij, l1_ji) < 1, the entries whose pass-2 factor multiplies a
  * nonzero remainder), "U1" [m][n], "A" [m][nnz]; entries follow gdg_problem's order (boundary data its
  * own).
- * "ls_deferred" [2] gives the number of line searches of each limiter pass that needed the bracketed
- * iteration (run by a separate kernel over a queue).  count must equal the array size.  Synchronises
+ * "ls_deferred" [2] gives the number of line searches of each limiter pass that FP32 did not settle
+ * (run by a separate kernel over a queue).  count must equal the array size.  Synchronises
  * the stream. */
 int gdg_debug_export(gdg_handle* h, const char* name, double* host_dst, int64_t count, void* stream);
 

@@ -1067,34 +1067,41 @@ __device__ __forceinline__ float ls_root_f32(const Dev& D, const double* U0, con
 
 // What psi's own rounding leaves open, relative to E: its terms are at most E in size, each good to an ulp
 // or so.
-constexpr double kPsiRounding = 2.220446049250313e-16;
+constexpr float kPsiRounding = 0x1p-52f;
 
 // A queued search: l_rho from the density bounds in closed form; psi(l_rho) >= 0, and l_rho is the answer, or
 // psi(0) < 0 (roundoff), and 0 is; else a feasible point within ls_tol, or psi's rounding, of the root in between.
 // Newton steps in FP64 from the FP32 root reach the rounding of psi in two or three evaluations; every
-// evaluated point narrows the bracket [a, b] of feasible and infeasible ends.  The search ends where the step
-// is at most half the tolerance, or where psi or the bracket is below psi's own rounding (then its sign, not its
-// size, is all there is): at that point when it is feasible, else at one just before it that is.  A step that
-// leaves the bracket, or does not settle in a few, hands over to the plain bracketed iteration (chord
-// root, tangent root from the infeasible end, and a bisection where the bracket has not halved), which is
-// also what a caller gets who allows fewer than 8 iterations.
+// evaluated point narrows the bracket [a, b] of feasible and infeasible ends.  The search ends at a feasible point whose root
+// estimate is within ls_tol / 2 or psi's rounding of it, or where the bracket is below ls_tol or twice that rounding (psi's
+// sign, not its size, is all there is then).  Every step goes a margin beyond the root estimate, so that its end is feasible
+// as a rule: a sixteenth of ls_tol or psi's rounding, doubled while points that close stay infeasible; the estimate itself is
+// good to the rounding.  (A first form stepped without a margin and then went back by the last step and ls_tol / 2 or the
+// rounding, in doubled strides: as many evaluations, but up to twice the error of the plain iteration.  Root mean square
+// errors in units of psi's rounding, of the plain iteration with the functions it had then, of that form and of this one: 0.53, 0.96
+// and 0.49 (Q3 vortex), 0.78, 1.17 and 0.67 (Q2 quadrants), 50, 67 and 9.4 (Q1 octants, where ls_tol is the larger).)
+// A step that leaves a wider bracket, or does not settle in eight, hands over to the plain bracketed iteration (chord
+// root, tangent root from the infeasible end, and a bisection where the bracket has not halved), whose iterations
+// ls_maxit counts and which is also what a caller gets who allows fewer than 8 of them.
 //
 // What bounds it is the length of the chain: every search is one thread, its evaluations follow one
 // another, and each is some 25 dependent FP64 operations of 64 clocks.  The plain iteration takes 20 to
-// 60 of them, this one about 4.  All of them go through one copy of the evaluation, chosen by a phase:
+// 60 of them, this one about 5.  All of them go through one copy of the evaluation, chosen by a phase:
 // lanes of a warp evaluate together whatever they do next, and the code a warp has to fetch cold, which
 // on small meshes takes longer than running it, stays short.  Per launch of k_lsfix, against the plain
-// iteration: 110 -> 24 us for 1,435 searches (Q2, 33 x 47 quads), 1,207 -> 238 us for 493,000 (Q1,
-// 48 x 40 x 44 hexahedra), 316 -> 66 us for 91,000 (Q2, 1024^2).
+// iteration: 110 -> 16 us for 1,435 searches (Q2, 33 x 47 quads), 1,207 -> 182 us for 493,000 (Q1,
+// 48 x 40 x 44 hexahedra), 316 -> 46 us for 91,000 (Q2, 1024^2).
 template <int DIM>
 __device__ __forceinline__ double line_search(const Dev& D, const double* U0, const double* A, double w, double rmin,
                                               double rmax, double smin) {
-  enum { kFull, kZero, kNewton, kBack, kChord, kTangent, kMiddle };
+  enum { kFull, kZero, kNewton, kChord, kTangent, kMiddle };
   // comparisons with the non-negative ends of the bracket, on the integer pipe
   auto above = [](double x, double y) { return __double_as_longlong(x) > __double_as_longlong(y); };
   const double l = ls_density(U0[0], sf::mul(w, A[0]), rmin, rmax);
   double a = 0.0, b = l, fa = 0.0, fb = 0.0, dfb = 0.0;
-  double t = l, t0 = 0.0, back = 0.0, width = 0.0, tn = 0.0;
+  double t = l, width = 0.0, tn = 0.0;
+  const float tol = to_f32(D.ls_tol);
+  float ef = 0.f, margin = 0.f;  // psi's rounding; how far beyond a root estimate the next step ends
   int phase = kFull, count = 0;
   for (;;) {
     double d;
@@ -1112,6 +1119,7 @@ __device__ __forceinline__ double line_search(const Dev& D, const double* U0, co
     if (phase == kZero) {
       if (!ok) return 0.0;
       fa = f;
+      ef = kPsiRounding * fmaxf(to_f32(U0[DIM + 1]), to_f32(fma(l * w, A[DIM + 1], U0[DIM + 1])));
       t = D.ls_maxit >= 8 ? to_f64(ls_root_f32<DIM>(D, U0, A, w, smin, l, f)) : 0.0;
       if (above(t, a) && above(b, t)) {
         phase = kNewton;
@@ -1127,32 +1135,19 @@ __device__ __forceinline__ double line_search(const Dev& D, const double* U0, co
         dfb = d;
       }
       if (phase == kNewton && d < 0.0) {
-        const double id = rcp64(d), step = __dmul_rn(f, id);
-        const double noise = abs_bits(__dmul_rn(kPsiRounding * id, fma(t * w, A[DIM + 1], U0[DIM + 1])));
-        if (!above(b - a, pmax(D.ls_tol, sf::mul_pow2(noise, 2)))) return a;
-        const double thr = pmax(sf::mul_pow2(D.ls_tol, -1), noise);
-        if (!above(abs_bits(step), thr)) {
-          if (ok) return t;
-          back = abs_bits(step) + thr;
-          t0 = t;
-          t = t0 - back;
-          if (!above(t, a)) return a;
-          phase = kBack;
-          count = 0;
-          continue;
-        }
-        t -= step;
+        // all that is compared, in FP32: the steps' sizes and psi's rounding, in units of t
+        const double id = rcp64(d);
+        const float size = fabsf(__fmul_rn(to_f32(f), to_f32(id))), noise = fabsf(__fmul_rn(ef, to_f32(id)));
+        if (!(to_f32(is_zero_bits(a) ? b : b - a) > fmaxf(tol, 2.f * noise))) return a;
+        const bool close = size <= fmaxf(0.5f * tol, noise);
+        if (ok && close) return t;
+        margin = fmaxf(close ? 2.f * margin : 0.f, fmaxf(0.0625f * fmaxf(noise, tol), 0x1p-52f * to_f32(t)));
+        t -= fma(f, id, to_f64(margin));
         if (above(t, a) && above(b, t) && ++count < 8) continue;
-      }
-      if (phase == kBack) {
-        if (ok) return t;
-        back = sf::mul_pow2(back, 2);
-        t = t0 - back;
-        if (!above(t, a)) return a;  // the bracket is no wider than what the step and the rounding leave open
-        if (++count < 3) continue;
+        if (!above(t, a) || !(to_f32(b - a) > fmaxf(tol, 4.f * noise))) return a;
       }
     }
-    if (phase <= kBack) {  // the Newton steps did not settle, or there is no start for them: the plain iteration
+    if (phase <= kNewton) {  // the Newton steps did not settle, or there is no start for them: the plain iteration
       count = 0;
       phase = kMiddle;
       width = 2.0 * (b - a);  // (the bisection below is for an iteration that has been run)
