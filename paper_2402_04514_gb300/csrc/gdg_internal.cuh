@@ -270,8 +270,10 @@ __device__ __forceinline__ double stage_tau(const Ctx& c) {
 // the local block is blockIdx.x.  Many: a batch; the block's instance is the last k with
 // start[k] <= blockIdx.x (binary search over the batch's per-kernel block offsets), its context is
 // copied from the device table into shared memory, and the local block is blockIdx.x - start[k].  Every
-// thread of the block must call get() before any thread leaves.
+// thread of the block must call get() before any thread leaves.  kSameLaunch: whether the stage's own arrays are written
+// by the launch that reads them (persistent.cu's source).
 struct One {
+  static constexpr bool kSameLaunch = false;
   Ctx c;
   __device__ __forceinline__ const Ctx& get(Ctx*, int* lb, int* nblk = nullptr) const {
     *lb = blockIdx.x;
@@ -285,7 +287,19 @@ struct One {
   }
 };
 
+// A value of the stage's own arrays (Scratch) that no thread of this kernel body writes: by the read-only path, which may move
+// ahead of the body's stores, where another launch wrote it; that path is defined for data that no thread of the launch
+// writes, so a launch that runs several bodies takes an ordinary load, which its grid-wide barriers order.
+template <class Src, class T>
+__device__ __forceinline__ T ld_stage(const T* p) {
+  if constexpr (Src::kSameLaunch)
+    return *p;
+  else
+    return __ldg(p);
+}
+
 struct Many {
+  static constexpr bool kSameLaunch = false;
   const Ctx* ctx;   // device [ninst]
   const int* start; // device [ninst + 1] first block of each instance, then the total
   int ninst;

@@ -98,8 +98,8 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
       else
         rhs[q] = S.RHSL[(size_t)q * n + i];
     }
-    // min / max of non-negative values on the integer pipe; every input of the loop is read-only in this
-    // kernel, so its loads take the read-only path and may move ahead of the stores of A.  The same pass
+    // min / max of non-negative values on the integer pipe; no thread of this body writes an input of the loop, so its
+    // loads take the read-only path where that is defined (ld_stage) and may move ahead of the stores of A.  The same pass
     // over I(i) gathers the two-hop aggregates of the relaxed bounds (step 3).
     const int e1 = D.sten_end[i];
     if (lim) {
@@ -115,11 +115,11 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
       const int j = __ldg(D.col + e);
       double Uj[M];
 #pragma unroll
-      for (int q = 0; q < M; ++q) Uj[q] = __ldg(U + (size_t)q * n + j);
+      for (int q = 0; q < M; ++q) Uj[q] = ld_stage<Src>(U + (size_t)q * n + j);
       if (lim) {
-        lo = pmin(lo, __ldg(S.agg + j));
-        hi = pmax(hi, __ldg(S.agg + n + j));
-        sl = pmin(sl, __ldg(S.agg + 2 * n + j));
+        lo = pmin(lo, ld_stage<Src>(S.agg + j));
+        hi = pmax(hi, ld_stage<Src>(S.agg + n + j));
+        sl = pmin(sl, ld_stage<Src>(S.agg + 2 * n + j));
       }
       bool same = true;
 #pragma unroll
@@ -132,7 +132,7 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
         continue;
       }
       quiet = false;
-      const double dl64 = __ldg(S.dL + e), mu = __ldg(D.mu + e), Nj = abs_bits(__ldg(S.N + j));
+      const double dl64 = ld_stage<Src>(S.dL + e), mu = __ldg(D.mu + e), Nj = abs_bits(ld_stage<Src>(S.N + j));
       if constexpr (MX) {
         // d^H - d^L from FP32 operands: every factor is symmetric in (i, j), so the same bits come out
         // of row j, and A_ji = -A_ij holds exactly

@@ -206,7 +206,7 @@ __device__ __forceinline__ void tau_body(const Src& src, int sliced) {
     double dsum = 0.0;
     const int e0 = D.rbeg[i], e1 = D.sten_end[i];
 #pragma unroll 4
-    for (int e = e0; e < e1; e += kEll) dsum += __ldg(dL + e);  // loads issued ahead of the in-order sum
+    for (int e = e0; e < e1; e += kEll) dsum += ld_stage<Src>(dL + e);  // loads issued ahead of the in-order sum
     for (int b = D.b_ptr[i], b1 = D.b_ptr[i + 1]; b < b1; ++b) dsum += dB[b];
     if (dsum > 0.0) val = sf::mul(sf::mul_pow2(D.mi[i], -1), rcp64(dsum));
   }

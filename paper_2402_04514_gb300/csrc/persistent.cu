@@ -18,6 +18,7 @@ namespace {
 // instance k with start[k] <= vb (the batch's block offsets for that kernel, computed for the persistent
 // block size), exactly as Many maps blockIdx.x.  Every thread of the block must call get().
 struct Virt {
+  static constexpr bool kSameLaunch = true;
   const Ctx* ctx;
   const int* start;
   int ninst;
