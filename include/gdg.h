@@ -216,7 +216,8 @@ int gdg_status(gdg_handle* h, int32_t* flags, int32_t clear, void* stream);
  * "dL" [nnz], "dB" [nb], "N" [n], "UL" [m][n], "rho_min" [n], "rho_max" [n], "s_min" [n], "l1" [nnz],
  * "l2" [nnz] (written only where min(l1_ij, l1_ji) < 1, the entries whose pass-2 factor multiplies a
  * nonzero remainder), "U1" [m][n], "A" [m][nnz]; entries follow gdg_problem's order (boundary data its
- * own).
+ * own).  gdg_max_dt leaves them alone; what a stage of order LOW, or HIGH, or of fewer passes does not work out has no
+ * defined value after it ("A" after order HIGH: the viscous part, of entries with c_ij != 0).
  * "ls_deferred" [2] gives the number of line searches of each limiter pass that FP32 did not settle
  * (run by a separate kernel over a queue).  count must equal the array size.  Synchronises
  * the stream. */

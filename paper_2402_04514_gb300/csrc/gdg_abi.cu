@@ -108,7 +108,7 @@ struct Arena {
   X(UB, double, m * nb) X(gB, double, m * nb) X(gI, double, m * nb)                                       \
   X(UL, double, m * n) X(RHSL, double, m * n) X(N, double, n) X(agg, double, 3 * n) X(A, double, m * nnz) \
   X(AB, double, m * nb) X(bounds, double, 3 * n) X(l1, double, nnz) X(l1B, double, nb) X(l2, double, nnz) \
-  X(l2B, double, nb) X(U1, double, m * n) X(rem, unsigned char, n) X(flags, unsigned, 4)                 \
+  X(l2B, double, nb) X(U1, double, m * n) X(Us, double, m * n) X(rem, unsigned char, n) X(flags, unsigned, 4) \
   X(tau, unsigned long long, 1)                                                                          \
   X(lsq, int2, nnz + nb) X(clk, gdg::Clock, 1)
 
@@ -662,7 +662,7 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   S.l2 = (double*)ptr(o_l2);
   S.l2B = (double*)ptr(o_l2B);
   S.U1 = (double*)ptr(o_U1);
-  S.Us = S.U1;
+  S.Us = (double*)ptr(o_Us);
   S.rem = (unsigned char*)ptr(o_rem);
   S.flags = (unsigned*)ptr(o_flags);
   S.lsq_n = S.flags + 2;
@@ -1064,14 +1064,29 @@ int gdg_debug_export(gdg_handle* h, const char* name, double* dst, int64_t count
   if (kind == 0 && per_entry) {  // device entry order back to the caller's
     for (int64_t r = 0; r < want / std::max<int64_t>(nnz, 1); ++r)
       for (int64_t q = 0; q < nnz; ++q) dst[r * nnz + h->eorig[q]] = tmp[r * NE + h->epos[q]];
-    if (nm == "A" && h->D.order == GDG_ORDER_LIMITED && h->D.passes > 0) {  // rows whose A is zero are not stored
+    if (nm == "A" && n > 0) {  // zeros that the element sweep does not store: whole rows, or entries between equal states
       std::vector<unsigned char> rem(h->ns);
-      if (n > 0 && (e = cudaMemcpy(rem.data(), h->S.rem, h->ns, cudaMemcpyDeviceToHost)) != cudaSuccess)
+      std::vector<int> sten(h->ns);
+      std::vector<double> Us((size_t)m * h->ns);
+      if ((e = cudaMemcpy(rem.data(), h->S.rem, h->ns, cudaMemcpyDeviceToHost)) != cudaSuccess ||
+          (e = cudaMemcpy(sten.data(), h->D.sten_end, sizeof(int) * h->ns, cudaMemcpyDeviceToHost)) != cudaSuccess ||
+          (e = cudaMemcpy(Us.data(), h->S.Us, sizeof(double) * Us.size(), cudaMemcpyDeviceToHost)) != cudaSuccess)
         return cuda_fail(e);
-      for (int64_t i = 0; i < n; ++i)
-        if (rem[node_slot(i, h->n_loc)] == 2)
-          for (int64_t q = h->row_ptr[i]; q < h->row_ptr[i + 1]; ++q)
+      for (int64_t i = 0; i < n; ++i) {
+        const int64_t t = node_slot(i, h->n_loc);
+        if (rem[t] != 2 && rem[t] != 3) continue;
+        for (int64_t q = h->row_ptr[i]; q < h->row_ptr[i + 1]; ++q) {
+          bool zero = rem[t] == 2;
+          if (!zero && h->epos[q] < sten[t]) {
+            const int64_t tj = node_slot(h->col[q], h->n_loc);
+            zero = true;
+            for (int64_t r = 0; r < m; ++r)
+              zero = zero && std::memcmp(&Us[r * h->ns + t], &Us[r * h->ns + tj], sizeof(double)) == 0;
+          }
+          if (zero)
             for (int64_t r = 0; r < m; ++r) dst[r * nnz + h->eorig[q]] = 0.0;
+        }
+      }
     }
   } else if (per_node) {
     for (int64_t r = 0; r < want / std::max<int64_t>(n, 1); ++r)

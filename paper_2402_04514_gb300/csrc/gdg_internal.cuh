@@ -182,9 +182,9 @@ struct Scratch {
   double* l2;      // [nnz] pass 2
   double* l2B;     // [nb]
   double* U1;      // [m][ns]
-  double* Us;      // [m][ns] the stage input by slots, from k_prim to k_high (in the place of U1, which comes later)
-  unsigned char* rem;  // [ns] from the element sweep: 2 where all of row i's A is zero and therefore not stored; then from
-                       // sweep C also 1 where the row has a pass-2 remainder (a symmetrised pass-1 factor below 1)
+  double* Us;      // [m][ns] the stage input by slots, from k_prim to k_high
+  unsigned char* rem;  // [ns] from the element sweep: 2 where all of row i's A is zero and therefore not stored, 3 with order HIGH,
+                       // which stores no zeros between equal states; then from sweep C also 1 where the row has a pass-2 remainder (a symmetrised pass-1 factor below 1)
   unsigned int* flags;
   unsigned int* lsq_n;  // [2] lengths of the deferred line-search queues of passes 1 and 2
   int2* lsq;            // [nnz + nb] deferred line searches of the current pass (ls_defer)

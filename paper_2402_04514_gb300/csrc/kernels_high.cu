@@ -251,7 +251,10 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
       }
     }
   }
-  if (D.order == GDG_ORDER_HIGH) return;
+  if (D.order == GDG_ORDER_HIGH) {
+    if (valid) S.rem[i] = 3;
+    return;
+  }
   __syncthreads();
   const int nl = D.n_loc;
   const int se = valid ? D.sten_end[i] : 0, r0 = valid ? D.rbeg[i] : 0, r1 = valid ? D.rend[i] : 0;
