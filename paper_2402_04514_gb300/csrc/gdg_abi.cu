@@ -103,7 +103,7 @@ struct Arena {
   X(mij, double, nnz) X(mu, double, nnz) X(mi, double, n) X(imi, double, n) X(ikm, double, n)             \
   X(rm, double, n) X(rp, double, n) X(muB, double, n) X(bptr, int, n + 1) X(bnorm, double, nb)           \
   X(bn, double, dim * nb) X(btype, int, nb) X(borig, int, nb) X(bnode, int, nb) X(minv, double, nel * nl * nl)             \
-  X(ee, int, ne) X(ei, int, ne) X(G, double, m * nnz) X(psi, double, nnz) X(barR, double, nnz) X(barS, double, nnz)          \
+  X(ee, int, ne) X(ei, int, ne)                                                                           \
   X(prim, double, gdg::NPRIM * n) X(dL, double, nnz) X(dB, double, nb) X(bbar, double, 2 * nb)            \
   X(UB, double, m * nb) X(gB, double, m * nb) X(gI, double, m * nb)                                       \
   X(UL, double, m * n) X(RHSL, double, m * n) X(N, double, n) X(agg, double, 3 * n) X(A, double, m * nnz) \
@@ -641,10 +641,11 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   Scratch& S = h->S;
   S.prim = (double*)ptr(o_prim);
   S.dL = (double*)ptr(o_dL);
-  S.G = (double*)ptr(o_G);
-  S.psi = (double*)ptr(o_psi);
-  S.barR = (double*)ptr(o_barR);
-  S.barS = (double*)ptr(o_barS);
+  // the edge sweep's per-entry values, which sweep A is the last to read, lie where later sweeps write theirs
+  S.G = (double*)ptr(o_A);
+  S.psi = (double*)ptr(o_lsq);
+  S.barR = (double*)ptr(o_l1);
+  S.barS = (double*)ptr(o_l2);
   S.dB = (double*)ptr(o_dB);
   S.bbar = (double*)ptr(o_bbar);
   S.UB = (double*)ptr(o_UB);

@@ -175,8 +175,8 @@ __device__ __forceinline__ void maxdt_body(const Src& src) {
   const double d = sf::mul(D.cnorm[e], lambda_pair<MX>(D, uL, P[PR_P * n + i], ir_i, P[PR_IP * n + i], P[PR_A * n + i],
                                                        P[PR_PME * n + i], uR, P[PR_P * n + j], ir_j, P[PR_IP * n + j],
                                                        P[PR_A * n + j], P[PR_PME * n + j]));
-  S.barR[e] = d;
-  S.barR[D.tr[e]] = d;
+  S.psi[e] = d;  // (l1, where barR lies, stays the last stage's)
+  S.psi[D.tr[e]] = d;
 }
 
 template <int DIM, bool MX, class Src>
@@ -199,7 +199,7 @@ __device__ __forceinline__ void tau_body(const Src& src, int sliced) {
   const Scratch& S = c.S;
   const Node nd = row_node(D, lb * blockDim.x + threadIdx.x, sliced);
   const int i = nd.t;
-  const double* dL = c.clk ? S.dL : S.barR;
+  const double* dL = c.clk ? S.dL : S.psi;
   const double* dB = c.clk ? S.dB : S.bbar;
   double val = INFINITY;
   if (nd.i >= 0) {
