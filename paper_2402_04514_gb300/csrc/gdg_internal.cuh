@@ -520,18 +520,6 @@ __device__ __forceinline__ float d2f_incr(double x, bool fz) {
   return __uint_as_float(r);
 }
 
-// FP32 -> FP64 by integer operations only: exact for normal numbers, zeros, infinities and NaN; an FP32
-// subnormal gives NaN (no caller produces one where a result is needed: the seeds below are normal, and
-// a NaN certificate fails).
-__device__ __forceinline__ double f2d_fast(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned sg = u & 0x80000000u, e = (u >> 23) & 0xffu, mt = u & 0x7fffffu;
-  unsigned hi = sg | ((e + 896u) << 20) | (mt >> 3);
-  if (e == 255u) hi = sg | 0x7ff00000u | (mt >> 3);
-  if (e == 0u) hi = mt ? 0x7ff80000u : sg;
-  return __hiloint2double((int)hi, (int)(mt << 29));
-}
-
 // |x| and min / max of non-negative doubles through their bit patterns (IEEE order of non-negative
 // numbers is the integer order), and x == +-0; all on the integer pipe.
 __device__ __forceinline__ double abs_bits(double x) {
@@ -539,10 +527,6 @@ __device__ __forceinline__ double abs_bits(double x) {
 }
 __device__ __forceinline__ bool same_bits(double x, double y) {
   return __double_as_longlong(x) == __double_as_longlong(y);
-}
-// x or'ed into a mask that stays zero while every x is +-0
-__device__ __forceinline__ void nonzero_bits(unsigned& mask, double x) {
-  mask |= ((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x);
 }
 __device__ __forceinline__ bool is_zero_bits(double x) { return (__double_as_longlong(x) << 1) == 0; }
 __device__ __forceinline__ bool is_one_bits(double x) { return __double_as_longlong(x) == 0x3ff0000000000000LL; }
@@ -930,20 +914,7 @@ __device__ __forceinline__ void ls_row(const Dev& D, LsRow<DIM>& c, const double
 }
 
 // psi(s) = eps(U0 + s A) - s_min rho(s)^gamma (the entropy constraint of the set B_i, Sec. 5.4,
-// eq. (BiSet), times rho^gamma); concave in s.
-template <int DIM>
-__device__ __forceinline__ double ls_psi(const Dev& D, const double* U0, const double* A, double s, double smin) {
-  double V[DIM + 2];
-#pragma unroll
-  for (int q = 0; q < DIM + 2; ++q) V[q] = fma(s, A[q], U0[q]);
-  if (!(V[0] > 0.0)) return -1.0;
-  const double m2 = dot_fp64<DIM>(V + 1, V + 1);
-  double irho;
-  double rg = rho_pow_gamma(D, V[0], &irho);
-  return fma(-smin, rg, fma(-sf::mul_pow2(m2, -1), irho, V[DIM + 1]));
-}
-
-// psi(s), computed as ls_psi computes it, and d psi / d s (the two share the state, rho^gamma and 1/rho).
+// eq. (BiSet), times rho^gamma), concave in s, and d psi / d s.
 template <int DIM>
 __device__ __forceinline__ double ls_psi_dpsi(const Dev& D, const double* U0, const double* A, double s, double smin,
                                               double* dpsi) {

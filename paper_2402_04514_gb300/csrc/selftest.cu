@@ -14,7 +14,7 @@ __global__ void k_math(int fn, int q, const double* __restrict__ x, double* __re
     case 1: y[i] = rootinv(v, root_q(q)); break;
     case 2: y[i] = 1.0 / v; break;
     case 3: y[i] = pow(v, -1.0 / q); break;
-    case 4: y[i] = f2d_fast(d2f_fast(v)); break;
+    case 4: y[i] = to_f64(d2f_fast(v)); break;
     case 5: y[i] = sqrt64(v); break;
     case 6: y[i] = sqrt(v); break;
     default: y[i] = 0.0;
@@ -114,7 +114,8 @@ __global__ void k_cert(Dev D, const double* __restrict__ in, double* __restrict_
   LsRow<DIM> c;
   ls_row<DIM>(D, c, U0, 0.0, INFINITY, smin);
   out[2 * k] = ls_certified<DIM>(D, c, A, d2f_fast(sv)) ? 1.0 : 0.0;
-  out[2 * k + 1] = ls_psi<DIM>(D, U0, A, sv, smin);
+  double dpsi;
+  out[2 * k + 1] = ls_psi_dpsi<DIM>(D, U0, A, sv, smin, &dpsi);  // as the deferred searches evaluate it
 }
 
 }  // namespace
