@@ -781,12 +781,6 @@ __device__ __forceinline__ double dot_fp64(const double* a, const double* b) {
   return s;
 }
 
-template <int DIM>
-__device__ __forceinline__ double internal_energy(const double* U) {
-  const double m2 = dot<DIM>(U + 1, U + 1);
-  return U[DIM + 1] - sf::mul_pow2(m2, -1) / U[0];
-}
-
 // In- and outflow boundary state (Sec. 4.1) from the interior state Ui, the data Ud and the outward unit
 // normal n: supersonic inflow (v.n < -a) takes the data, supersonic outflow (v.n >= a) the interior state
 // (eq. (eq:supersonic_inoutflow)); in between, the characteristic variables of eq. (eq:characteristics),

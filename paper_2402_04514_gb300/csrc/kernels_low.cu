@@ -100,24 +100,35 @@ __global__ void __launch_bounds__(kThreads) k_prim(Src src) {
   prim_body<DIM, MX, Src>(src);
 }
 
-// d_i^{d,k} = |c_i^{d,k}| lambda_max^+(U_i, U^{d,k}, n_i^k) of boundary entry b (Sec. 4.2,
-// eq. (eq:dij_low_order_modified); interior state on the left), from node i's primitives.
+// Boundary entry b of a stage: the unit normal, the interior and the boundary state, their m.n, v.n and pressures, and
+// d_i^{d,k} = |c_i^{d,k}| lambda_max^+(U_i, U^{d,k}, n_i^k) (Sec. 4.2, eq. (eq:dij_low_order_modified); interior state on
+// the left).
+template <int DIM>
+struct Side {
+  double n[DIM], Ui[DIM + 2], UB[DIM + 2], mnL, mnR, uL, uR, pL, pB, d;
+};
 template <int DIM, bool MX>
-__device__ __forceinline__ double boundary_viscosity(const Dev& D, int b, const double* Ui, const double* bdata,
-                                                     double irho_i, double p_i, double ip_i, double a_i,
-                                                     double pme_i) {
-  constexpr int M = DIM + 2;
-  double nv[DIM], UB[M];
+__device__ __forceinline__ void boundary_side(const Ctx& c, int b, Side<DIM>& o) {
+  const Dev& D = c.D;
+  const double* P = c.S.prim;
+  const size_t n = D.ns, nb = D.nb;
+  const int i = D.bnode[b];
+  load_state<DIM>(c.S.Us, D.ns, i, o.Ui);
+  const double irL = P[PR_IRHO * n + i];
+  o.pL = P[PR_P * n + i];
 #pragma unroll
-  for (int k = 0; k < DIM; ++k) nv[k] = D.bn[(size_t)k * D.nb + b];
-  boundary_state<DIM>(D, b, Ui, bdata, nv, UB);
-  double irB = 1.0 / UB[0];
-  double pB = sf::mul(D.gm1, internal_energy<DIM>(UB));
-  const double uL = dot<DIM>(Ui + 1, nv), uR = dot<DIM>(UB + 1, nv);
+  for (int k = 0; k < DIM; ++k) o.n[k] = D.bn[(size_t)k * nb + b];
+  boundary_state<DIM>(D, b, o.Ui, c.bdata, o.n, o.UB);
+  const double irB = rcp64(o.UB[0]);
+  o.pB = sf::mul(D.gm1, fma(-sf::mul_pow2(dot<DIM>(o.UB + 1, o.UB + 1), -1), irB, o.UB[DIM + 1]));
+  o.mnL = dot<DIM>(o.Ui + 1, o.n);
+  o.mnR = dot<DIM>(o.UB + 1, o.n);
+  o.uL = sf::mul(o.mnL, irL);
+  o.uR = sf::mul(o.mnR, irB);
   double ipB, aB, pmeB;
-  prim_of<MX>(D, UB[0], irB, pB, &ipB, &aB, &pmeB);
-  return sf::mul(D.bnorm[b], lambda_pair<MX>(D, sf::mul(uL, irho_i), p_i, irho_i, ip_i, a_i, pme_i, sf::mul(uR, irB),
-                                             pB, irB, ipB, aB, pmeB));
+  prim_of<MX>(D, o.UB[0], irB, o.pB, &ipB, &aB, &pmeB);
+  o.d = sf::mul(D.bnorm[b], lambda_pair<MX>(D, o.uL, o.pL, irL, P[PR_IP * n + i], P[PR_A * n + i], P[PR_PME * n + i], o.uR,
+                                            o.pB, irB, ipB, aB, pmeB));
 }
 
 // Block minimum of val, then one 64-bit atomicMin per block on the bit pattern (positive doubles order
@@ -141,7 +152,6 @@ __device__ __forceinline__ void block_min_to(double val, unsigned long long* dst
 // the row sums at Q2 33 x 47.
 template <int DIM, bool MX, class Src>
 __device__ __forceinline__ void maxdt_body(const Src& src) {
-  constexpr int M = DIM + 2;
   __shared__ Ctx sctx;
   int lb;
   const Ctx& c = src.get(&sctx, &lb);
@@ -153,11 +163,9 @@ __device__ __forceinline__ void maxdt_body(const Src& src) {
   const unsigned slot = lb * blockDim.x + threadIdx.x, nbs = boundary_slots(D.nb);
   if (slot < nbs) {
     if (slot >= (unsigned)D.nb) return;
-    const int i = D.bnode[slot];
-    double Ui[M];
-    load_state<DIM>(S.Us, D.ns, i, Ui);
-    S.bbar[slot] = boundary_viscosity<DIM, MX>(D, (int)slot, Ui, c.bdata, P[PR_IRHO * n + i], P[PR_P * n + i],
-                                               P[PR_IP * n + i], P[PR_A * n + i], P[PR_PME * n + i]);
+    Side<DIM> side;
+    boundary_side<DIM, MX>(c, (int)slot, side);
+    S.bbar[slot] = side.d;
     return;
   }
   const unsigned k = slot - nbs;
@@ -244,28 +252,15 @@ __device__ __noinline__ void boundary_entry(const Ctx& c, int b) {
   constexpr int M = DIM + 2;
   const Dev& D = c.D;
   const Scratch& S = c.S;
-  const size_t n = D.ns, nb = D.nb;
-  const int i = D.bnode[b];
-  const double* P = S.prim;
-  double Ui[M], nv[DIM], UB[M];
-  load_state<DIM>(S.Us, D.ns, i, Ui);
-  const double irho_i = P[PR_IRHO * n + i], p_i = P[PR_P * n + i];
-#pragma unroll
-  for (int k = 0; k < DIM; ++k) nv[k] = D.bn[(size_t)k * nb + b];
-  boundary_state<DIM>(D, b, Ui, c.bdata, nv, UB);
-  const double irB = rcp64(UB[0]);
-  const double pB = sf::mul(D.gm1, fma(-sf::mul_pow2(dot<DIM>(UB + 1, UB + 1), -1), irB, UB[DIM + 1]));
-  const double mnL = dot<DIM>(Ui + 1, nv), mnR = dot<DIM>(UB + 1, nv);
-  const double uL = sf::mul(mnL, irho_i), uR = sf::mul(mnR, irB);
-  const double cnm = D.bnorm[b];
-  double ipB, aB, pmeB;
-  prim_of<MX>(D, UB[0], irB, pB, &ipB, &aB, &pmeB);
-  const double d = sf::mul(cnm, lambda_pair<MX>(D, uL, p_i, irho_i, P[PR_IP * n + i], P[PR_A * n + i],
-                                                P[PR_PME * n + i], uR, pB, irB, ipB, aB, pmeB));
+  const size_t nb = D.nb;
+  Side<DIM> o;
+  boundary_side<DIM, MX>(c, b, o);
+  const double cnm = D.bnorm[b], d = o.d;
+  const double *Ui = o.Ui, *UB = o.UB;
   S.dB[b] = d;
   double fi[M], fB[M], Ub[M];
-  flux_n<DIM>(Ui, nv, mnL, uL, p_i, fi);
-  flux_n<DIM>(UB, nv, mnR, uR, pB, fB);
+  flux_n<DIM>(Ui, o.n, o.mnL, o.uL, o.pL, fi);
+  flux_n<DIM>(UB, o.n, o.mnR, o.uR, o.pB, fB);
   const double t = sf::mul(sf::mul_pow2(cnm, -1), rcp64(d));
 #pragma unroll
   for (int q = 0; q < M; ++q) {
