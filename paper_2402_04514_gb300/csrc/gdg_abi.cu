@@ -19,10 +19,11 @@ using gdg::Scratch;
 
 namespace {
 
+// f(begin, end) over [0, count) by all cores, grain at least of the range to each.
 template <class F>
-void parallel_for(int64_t count, F&& f) {
+void parallel_for(int64_t count, F&& f, int64_t grain = 65536) {
   unsigned hw = std::thread::hardware_concurrency();
-  int nt = (int)std::min<int64_t>(std::max(1u, std::min(hw, 32u)), std::max<int64_t>(1, count / 65536));
+  int nt = (int)std::min<int64_t>(std::max(1u, std::min(hw, 32u)), std::max<int64_t>(1, count / grain));
   if (nt <= 1) {
     f(0, count);
     return;
@@ -521,17 +522,28 @@ int gdg_setup(const gdg_problem* P, gdg_handle** out) {
   });
   // canonical stencil edges (i < j, c_ij != 0) in ELL order: consecutive threads of the edge sweep take
   // the same entry of the rows of consecutive elements, so their per-entry writes are contiguous
-  std::vector<std::pair<int, int>> edges;
-  edges.reserve(nnz / 2 + 1);
-  for (int64_t i = 0; i < n; ++i)
-    for (int q = h->row_ptr[i]; q < h->row_ptr[i + 1]; ++q)
-      if (cnorm[q] > 0.0 && h->col[q] > i) edges.emplace_back(h->epos[q], (int)i);
-  std::sort(edges.begin(), edges.end());
-  std::vector<int> edge_e(edges.size()), edge_i(edges.size());
-  for (size_t k = 0; k < edges.size(); ++k) {
-    edge_e[k] = edges[k].first;
-    edge_i[k] = slot[edges[k].second];
-  }
+  // (listed slice by slice, counted first: sorted as they come, by all cores)
+  const int64_t nslice = (int64_t)EL.sbase.size() - 1;
+  auto slice_edges = [&](int64_t sl, auto&& take) {
+    const int64_t g = sl / nl, l = sl % nl, width = (EL.sbase[(size_t)sl + 1] - EL.sbase[(size_t)sl]) / gdg::kEll;
+    for (int64_t k = 0; k < width; ++k)
+      for (int64_t E = g * gdg::kEll; E < std::min(nel, (g + 1) * gdg::kEll); ++E) {
+        const int64_t i = E * nl + l, q = h->row_ptr[i] + k;
+        if (q < sten_end[i] && h->col[q] > i) take(q, i);
+      }
+  };
+  std::vector<int64_t> first((size_t)nslice + 1, 0);
+  parallel_for(nslice, [&](int64_t b, int64_t e) {
+    for (int64_t sl = b; sl < e; ++sl) slice_edges(sl, [&](int64_t, int64_t) { ++first[(size_t)sl + 1]; });
+  }, 2048);
+  for (int64_t sl = 0; sl < nslice; ++sl) first[(size_t)sl + 1] += first[(size_t)sl];
+  std::vector<int> edge_e((size_t)first[(size_t)nslice]), edge_i(edge_e.size());
+  parallel_for(nslice, [&](int64_t b, int64_t e) {
+    for (int64_t sl = b; sl < e; ++sl) {
+      size_t k = (size_t)first[(size_t)sl];
+      slice_edges(sl, [&](int64_t q, int64_t i) { edge_e[k] = h->epos[q], edge_i[k++] = slot[i]; });
+    }
+  }, 2048);
   const int64_t ne = (int64_t)edge_e.size();
   // the boundary entries in the order of their nodes' slots, the caller's order within a node
   std::stable_sort(border.begin(), border.end(),
