@@ -2,13 +2,14 @@
 
 Bytes: every array a kernel must read is read once and every array it writes is written once (per-entry
 arrays of nnz entries, per-node arrays of n nodes); neighbour states are counted once per node, not per
-entry (an ideal cache).  FP64 operations: the arithmetic of the method as the kernels state it, counted
-per stencil entry (c_ij != 0), per CSR entry and per node, with add/sub/mul = 1, fused multiply-add = 2,
-and division, square root and power = 1 each (the usual floating-point operation count; their cost in
-hardware is several to ~100 FMA issue slots, which is why the sweep is bound by arithmetic: the FP64 pipe
-and, for the products the kernels move there, the integer pipe).
-The line-search counts assume no bracketing iteration (the common case); iterations add work that is
-not counted, so the FP64 fraction reported is a lower bound.
+entry (an ideal cache), and what a kernel reads back of its own output is not counted.  FP64 operations: the
+arithmetic as the kernels state it for states of which no two agree, counted per undirected edge, per stencil
+entry (c_ij != 0), per pair of nodes of an element, per node and per boundary entry, with add/sub/mul = 1, fused
+multiply-add = 2, and division, square root and power = 1 each (the usual floating-point operation count; their
+cost in hardware is several to ~100 FMA issue slots, which is why the sweep is bound by arithmetic: the FP64 pipe
+and, for the products the kernels move there, the integer pipe).  FP32 work (the line searches' certificates) is not
+counted, nor what depends on the data: the deferred line searches, and the second pass of rows with a
+remainder, so that the FP64 fraction reported is a lower bound.
 """
 from __future__ import annotations
 
@@ -41,21 +42,24 @@ class Counts:
 
 def bytes_per_launch(c: Counts) -> dict:
     m, d, n, nnz, s, nb, nl = c.m, c.dim, c.n, c.nnz, c.nnz_s, c.nb, c.n_loc
-    NPRIM = 6
-    rowptr = 4 * (n + 1)
-    ent_geom = nnz * (4 + 8) + s * 8 * d  # col, |c| of every entry; n_ij of stencil entries
+    edge_geom = (s // 2) * (4 * 4 + 8 * (1 + d))  # entry, row, column, transpose; |c| and n_ij of one of the two entries
+    side_geom = nb * (3 * 4 + 8 * (1 + d))  # node, type, caller's index; |c| and normal of a boundary entry
+    pairs = n * (nl - 1) // 2  # of nodes of one element
     return dict(
-        prim=8 * m * n + 8 * NPRIM * n,
-        maxdt=8 * m * n + 8 * 4 * n + rowptr + ent_geom + 8 * n,
-        edge=(s // 2) * (4 * 2 + 4 + 4) + s * 8 * (1 + d) + 8 * (m + 5) * n + s * 8 * (m + 3),
-        low=8 * m * n + 8 * 3 * n + rowptr + nnz * (4 + 8) + s * (4 + 8 * (m + 3) + 8 * m)
-        + 8 * (2 * m + 1 + 3) * n + 8 * 3 * nb,
-        high=8 * m * n * 2 + 8 * n + rowptr + nnz * (4 + 8 + 8 + 8) + 8 * s * 2 + 8 * n * nl
-        + 8 * 3 * n * 2 + 8 * m * n + 8 * n * 3 + 8 * (m + 1) * nnz + 8 * (m + 1) * nb,
-        limit2=rowptr + nnz * (4 + 8 + 8 * m) + 8 * m * n * 2 + 8 * 3 * n + 8 * 2 * n + 8 * nnz,
-        final=rowptr + nnz * (4 + 8 * 2 + 8 * m) + 8 * m * n * 3 + 8 * n,
-        lsfix=0,  # the deferred line searches: a data-dependent handful of entries, not counted
-        tau=rowptr + 8 * nnz + 8 * n + 8 * (m + 6) * nb,
+        prim=8 * n * (m + m + 7),  # U -> U by slots, seven primitives
+        maxdt=edge_geom + 8 * n * (d + 5) + 8 * s + side_geom + 8 * nb,
+        # d, G, the indicator's term, rho and s~ of the bar state at both entries; a boundary entry's state, two
+        # fluxes, d and bar state
+        edge=edge_geom + 8 * n * (m + 7) + 8 * s * (m + 4) + side_geom + 8 * nb * (3 * m + 3),
+        low=n * 12 + 8 * n * (m + 4 + 1) + s * (4 + 8 * (m + 4)) + 8 * n * (2 * m + 4) + 8 * nb * (3 * m + 1),
+        # the rows' states, right-hand sides, U^L, aggregates, bounds, N and factors of the bounds and of P; M_K^-1;
+        # column, d, mu of the stencil; m_ij and transpose of an element's pairs; A and the factors
+        high=n * 17 + 8 * n * (3 * m + 3 + 3 + 1 + 2 + 1) + 8 * n * nl + 4 * nnz + 16 * s + 12 * pairs + 8 * nnz * (m + 1)
+        + 8 * nb * (2 * m + 5),
+        limit2=n * 14 + 8 * n * (2 * m + 1) + nnz * (4 + 8 * (m + 1)) + 8 * nb * (m + 1),
+        final=8 * m * n * 3 + n,
+        lsfix=0,  # the deferred line searches: data-dependent, not counted
+        tau=n * (12 + 8) + 8 * s + 8 * nb,
         clock=0,
         axpy=8 * m * n * 3,
     )
@@ -64,36 +68,34 @@ def bytes_per_launch(c: Counts) -> dict:
 def quiet_bytes_per_launch(c: Counts) -> dict:
     """bytes_per_launch of a mesh on which every state is the same: the edge sweep stores d_ij alone, sweep A reads nothing else
     of an entry but its column, the element sweep writes bounds and factors but no A, and sweep C reads no entry."""
-    m, d, n, nnz, s = c.m, c.dim, c.n, c.nnz, c.nnz_s
-    rowptr = 4 * (n + 1)
+    m, n, nnz, s, nb = c.m, c.n, c.nnz, c.nnz_s, c.nb
     out = bytes_per_launch(c)
-    out["edge"] = (s // 2) * (4 * 4 + 8 * (1 + d)) + 8 * (m + 5) * n + s * 8
-    out["low"] = 8 * m * n + 8 * 4 * n + rowptr + s * (4 + 8) + 8 * (2 * m + 1 + 3) * n
-    out["high"] = 8 * m * n * 2 + rowptr + s * 4 + 8 * 3 * n * 2 + 8 * n + 8 * nnz + n
-    out["limit2"] = rowptr + 8 * m * n * 2 + 2 * n
-    out["final"] = 8 * m * n * 3 + n
+    out["edge"] -= 8 * s * (m + 3)
+    out["low"] -= 8 * s * (m + 3)
+    out["high"] = n * 17 + 8 * n * (2 * m + 3 + 3 + 1 + 2) + 4 * s + 8 * nnz + 8 * nb * (2 * m + 5)
+    out["limit2"] = n * 14 + 8 * n * (2 * m + 1) + 8 * nb * (m + 1)
     return out
 
 
 def flops_per_launch(c: Counts) -> dict:
-    m, d, n, nnz, s, nb, nl = c.m, c.dim, c.n, c.nnz, c.nnz_s, c.nb, c.n_loc
-    lam = 28  # wave-speed bound from the per-node primitives
-    vel = 2 * (2 * d) + 2  # two normal velocities
+    m, d, n, s, nb, nl = c.m, c.dim, c.n, c.nnz_s, c.nb, c.n_loc
+    pairs = n * (nl - 1) // 2
+    lam = 23  # wave-speed bound from the stored primitives
+    vel = 4 * d  # two normal momenta and velocities
     flux = 2 * (3 * d + 2)  # f(U_i) n and f(U_j) n
-    ls = 2 * m + (3 * d + 3) + 3  # U0 + l P, eps, s_min rho^gamma (one psi evaluation)
-    edge_pair = vel + lam + 2 + flux + 2 + m + 4 * m + (3 * d + 3 + 2)  # per undirected stencil edge
-    low_entry = 1 + 4 * m + 3  # row sums of d, G and the entropy flux
-    low_node = 3 * m + 3 + 3 + 1 + 3 * d + 4 * m + 5 * m + 1
+    edge_pair = vel + lam + 1 + d + 4 + flux + 1 + 4 * m + 3 + (2 * d + 7)  # d_ij, G, W, the indicator's term, s~ of the bar state
+    side = 4 * d + 1 + (2 * d + 3) + vel + 5 + lam + 1  # a boundary entry's state, its primitives and d
+    low_node = 4 + 1 + 4 * m + (2 + d + 2 * d - 1 + 6 + 3 * d + 2) + 4 * m + 2
     return dict(
-        edge=(s // 2) * edge_pair,
-        prim=n * (1 + 3 * d + 3 + 1 + 2 + 3 + 1 + 2),
-        maxdt=s * (vel + lam + 2) + n * 3 + nb * (lam + vel + 10),
-        low=s * low_entry + n * low_node + nb * (vel + lam + flux + 11 * m + 10),
-        high=s * (4 + 3 * m) + n * (2 * nl * m + m + 3) + nnz * (4 * m + m + ls) + nb * (3 * m + ls),
-        limit2=nnz * (2 * m + 2 + m + ls) + n * 2 * m + nb * (2 * m + m + 2 + ls),
-        final=nnz * (2 + 2 * m) + n * 3 * m + nb * (2 + 2 * m),
+        edge=(s // 2) * edge_pair + nb * (side + flux + 3 + 7 * m + 2 * d + 5),
+        prim=n * (2 * d + 13),
+        maxdt=(s // 2) * (vel + lam + 1) + nb * side,
+        low=s * (4 * m + 2) + n * low_node + nb * (5 * m + 1),
+        high=s * (4 * m + 5) + pairs * 3 * m + n * (2 * nl * m + m + 3 + (2 * d + 8)) + nb * (5 * m + 3),
+        limit2=c.nnz * 2 * m + n * 2 * m + nb * 2 * m,
+        final=n * 3 * m,
         lsfix=0,
-        tau=nnz + 2 * n + nb * (lam + vel + 10),
+        tau=s + 3 * n + nb,
         clock=0,
         axpy=3 * m * n,
     )
