@@ -340,7 +340,8 @@ typedef struct {
   int32_t lsfix_slots;
   int32_t row_slices;  // bits 1 << GDG_K_{MAXDT,LOW,LIMIT2,FINAL,TAU}: that kernel's threads take their rows in
                        // the entry storage's slice order (a warp takes one local index of 32 consecutive
-                       // elements) instead of node order; default: all five
+                       // elements) instead of node order; default: all five.  MAXDT: the row sums of gdg_max_dt
+                       // (its wave speeds go by edges)
 } gdg_schedule;
 int gdg_autotune(gdg_handle* h, double* U, double* T1, double* T2, const double* bdata, int32_t trials,
                  void* stream);

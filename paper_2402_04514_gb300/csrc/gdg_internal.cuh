@@ -364,7 +364,8 @@ inline Sched default_sched() {
 
 // Row slots of a one-thread-per-row kernel: in node order slot t is row t; in ELL slice order slot t is
 // lane t % kEll of slice t / kEll = g n_loc + l, the row of local index l of element g kEll + t % kEll, so
-// that a warp's per-entry loads are contiguous (the nodes' own arrays are then read n_loc apart).
+// that a warp's loads of entries and of the library's own per-node arrays are contiguous (in node order both are
+// spread over slices; the caller's arrays, which the last writer of a stage takes, are contiguous then).
 __host__ __device__ inline long long row_slots(const Dev& D, bool sliced) {
   return sliced ? (long long)D.ns : (long long)D.n;
 }

@@ -356,8 +356,8 @@ __device__ __forceinline__ void high_sweep(const Src& src, int eb) {
 
 // The element sweep of each path as its own kernel with its own register budget.  Its loads, FP64 chains and 64-bit
 // integer chains leave the issue slots half empty at 27 warps per SM, so a few spills are worth a fourth 288-thread
-// block: in us per launch at 72, 56 and 48 registers 1,384, 1,231 and 1,185 (Q2 1024^2), 133, 99 and 104 (Q3 96^2), 240, 238
-// and 254 (Q1 512^2), 380, 372 and 357 (Q1 48 x 40 x 44); the mixed path 300, 261 and 242 (Q2 384^2).
+// block: in us per launch at 72, 56 and 48 registers 1,412, 1,268 and 1,211 (Q2 1024^2), 140, 109 and 114 (Q3 96^2), 239, 233
+// and 252 (Q1 512^2), 390, 379 and 370 (Q1 48 x 40 x 44); the mixed path 302, 261 and 241 (Q2 384^2).
 template <int DIM, class Src>
 __global__ void __maxnreg__(56) k_high(Src src, int eb) {
   chain_begin();

@@ -387,7 +387,7 @@ __device__ __forceinline__ void edge_body(const Src& src) {
 }
 
 // Two 512-thread blocks per SM (64 registers, a few bytes of spills): the integer-pipe products of the
-// sweep want resident warps to hide their latency (2.18 ms per launch at Q2 1024^2).
+// sweep want resident warps to hide their latency.
 template <int DIM, bool MX, class Src>
 __global__ void __launch_bounds__(kThreads, 2) k_edge(const __grid_constant__ Src src) {
   chain_begin();
