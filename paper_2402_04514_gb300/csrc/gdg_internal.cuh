@@ -1062,9 +1062,10 @@ constexpr float kPsiRounding = 0x1p-52f;
 // rounding, in doubled strides: as many evaluations, but up to twice the error of the plain iteration.  Root mean square
 // errors in units of psi's rounding, of the plain iteration with the functions it had then, of that form and of this one: 0.53, 0.96
 // and 0.49 (Q3 vortex), 0.78, 1.17 and 0.67 (Q2 quadrants), 50, 67 and 9.4 (Q1 octants, where ls_tol is the larger).)
-// A step that leaves a wider bracket, or does not settle in eight, hands over to the plain bracketed iteration (chord
-// root, tangent root from the infeasible end, and a bisection where the bracket has not halved), whose iterations
-// ls_maxit counts and which is also what a caller gets who allows fewer than 8 of them.
+// A step that leaves a wider bracket, or does not settle in eight, or a psi so flat that its rounding is a sixteenth of the
+// root or more, or no feasible point but 0 found, hands over to the plain bracketed iteration (chord root, tangent
+// root from the infeasible end, and a bisection where the bracket has not halved), whose iterations ls_maxit
+// counts and which is also what a caller gets who allows fewer than 8 of them.
 //
 // What bounds it is the length of the chain: every search is one thread, its evaluations follow one
 // another, and each is some 25 dependent FP64 operations of 64 clocks.  The plain iteration takes 20 to
@@ -1120,13 +1121,17 @@ __device__ __forceinline__ double line_search(const Dev& D, const double* U0, co
         // all that is compared, in FP32: the steps' sizes and psi's rounding, in units of t
         const double id = rcp64(d);
         const float size = fabsf(__fmul_rn(to_f32(f), to_f32(id))), noise = fabsf(__fmul_rn(ef, to_f32(id)));
-        if (!(to_f32(is_zero_bits(a) ? b : b - a) > fmaxf(tol, 2.f * noise))) return a;
-        const bool close = size <= fmaxf(0.5f * tol, noise);
-        if (ok && close) return t;
-        margin = fmaxf(close ? 2.f * margin : 0.f, fmaxf(0.0625f * fmaxf(noise, tol), 0x1p-52f * to_f32(t)));
-        t -= fma(f, id, to_f64(margin));
-        if (above(t, a) && above(b, t) && ++count < 8) continue;
-        if (!above(t, a) || !(to_f32(b - a) > fmaxf(tol, 4.f * noise))) return a;
+        bool end = !(to_f32(is_zero_bits(a) ? b : b - a) > fmaxf(tol, 2.f * noise));
+        const bool flat = noise > 0.0625f * to_f32(t);
+        if (!end && !flat) {
+          const bool close = size <= fmaxf(0.5f * tol, noise);
+          if (ok && close) return t;
+          margin = fmaxf(close ? 2.f * margin : 0.f, fmaxf(0.0625f * fmaxf(noise, tol), 0x1p-52f * to_f32(t)));
+          t -= fma(f, id, to_f64(margin));
+          if (above(t, a) && above(b, t) && ++count < 8) continue;
+          end = (close && !above(t, a)) || !(to_f32(b - a) > fmaxf(tol, 4.f * noise));
+        }
+        if (end && !flat && !is_zero_bits(a)) return a;
       }
     }
     if (phase <= kNewton) {  // the Newton steps did not settle, or there is no start for them: the plain iteration

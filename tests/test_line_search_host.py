@@ -57,3 +57,15 @@ def test_line_search_ends_at_the_rounding_of_psi(tmp_path, name):
     out = subprocess.run([exe, data], capture_output=True, text=True)
     print(out.stdout)
     assert out.returncode == 0, out.stdout + out.stderr
+
+
+def test_flat_directions_are_not_given_up(tmp_path):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None or not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h")):
+        pytest.skip("no C++ compiler or CUDA headers")
+    exe = str(tmp_path / "check")
+    subprocess.run([cxx, "-O2", "-std=c++17", "-w", "-ffp-contract=off", "-I" + os.path.join(CUDA, "include"),
+                    os.path.join(HERE, "flat_search_check.cpp"), "-o", exe], check=True)
+    out = subprocess.run([exe], capture_output=True, text=True)
+    print(out.stdout)
+    assert out.returncode == 0, out.stdout + out.stderr
